@@ -123,9 +123,9 @@ struct VolDev {
     uint32_t mrf_max;         // step limit, 0 = off
     uint32_t mrf_tiles;       // k_mrf_stats tiles of MRF_TILE octets (8 x-consecutive voxels)
     uint32_t mrf_tbase;       // first flat k_mrf_stats tile
-    uint32_t mrf_ctiles;      // k_mrf_step tiles: MRF_TX octets x MRF_TY rows, all of z
-    uint32_t mrf_cbase;       // first flat k_mrf_step tile
-    uint32_t mrf_vec;         // 1: X % 8 == 0 and the input 16-byte aligned (octets load as uint4)
+    uint32_t mrf_ctiles;      // k_mrf_step tiles of a plane (MRF_TILE octets of it)
+    uint32_t mrf_align;       // alignment of every octet of input and buffers: 16 (X % 8 == 0), 4 (X even) or 2 bytes
+    uint64_t mrf_ubase;       // first flat k_mrf_step unit (plane of a tile, z fastest)
 };
 
 // The distance-map kernels and their work items.  A volume takes the fused
@@ -142,9 +142,7 @@ enum DtKernel : int {
     DT_NK = 6,
 };
 constexpr int DZ_ELEMS = 8192;   // k_dist_z shared stack entries per block
-constexpr int MRF_TILE = 256;    // octets per k_mrf_stats tile (one per thread)
-constexpr int MRF_TX = 32;       // k_mrf_step tile: octets along x (one warp) ...
-constexpr int MRF_TY = 8;        // ... times rows, walked down z
+constexpr int MRF_TILE = 256;    // octets per k_mrf_stats and k_mrf_step tile (one per thread)
 constexpr uint32_t MRF_MAX_ITER = 1000;
 
 // Batch header, followed in memory by VolDev[nvol].
@@ -162,7 +160,7 @@ struct BatchHdr {
     uint32_t cl_items;   // closing dilation items over the batch
     uint32_t dt_items[DT_NK]; // distance-map items per DtKernel over the batch
     uint32_t mrf_tiles;       // k_mrf_stats tiles over the batch
-    uint32_t mrf_ctiles;      // k_mrf_step tiles over the batch
+    uint64_t mrf_units;       // k_mrf_step units over the batch
     uint32_t row_tile;        // rows per row tile: ROW_TILE, or down to ROW_TILE_MIN
                               // so that a batch with few rows still fills the GPU
     VolDev vol[1];       // nvol entries

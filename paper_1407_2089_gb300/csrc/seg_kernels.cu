@@ -2802,8 +2802,6 @@ __global__ void __launch_bounds__(ROW_TILE) k_erode(const BatchHdr *__restrict__
 // Delta is the smallest gap between two distinct input levels.  One tile is
 // MRF_TILE octets (8 x-consecutive voxels of a row) of one volume.
 
-__device__ __forceinline__ int mrf_sgn(int32_t d) { return (d > 0) - (d < 0); }
-
 // Block sum of one uint64 per thread (MRF_TILE threads); thread 0 gets it.
 __device__ __forceinline__ unsigned long long mrf_block_sum(unsigned long long v, unsigned long long *red) {
 #pragma unroll
@@ -2877,7 +2875,7 @@ __global__ void __launch_bounds__(MRF_TILE) k_mrf_stats(const BatchHdr *__restri
         const uint32_t row = o / OX, x0 = 8 * (o % OX), y = row % Y;
         const uint16_t *r0 = V.mrf_in + (size_t)row * X + x0;
         const uint32_t n = min(8u, X - x0);
-        const bool vec = n == 8u && V.mrf_vec;  // (mrf_buf is always aligned)
+        const bool vec = V.mrf_align == 16u;
         int32_t c[8];
         mrf_load8(r0, vec, n, c);
         for (uint32_t j = 0; j < n; ++j) {  // most levels are already marked: test before setting
@@ -2979,157 +2977,259 @@ __global__ void k_mrf_prep(const BatchHdr *__restrict__ h) {
     }
 }
 
-// Octet helpers of the step kernel: 8 voxels packed two to a word.
-__device__ __forceinline__ uint4 mrf_oct(const uint16_t *p, bool vec, uint32_t n) {
-    if (vec) return *reinterpret_cast<const uint4 *>(p);
-    uint32_t w[4] = {0u, 0u, 0u, 0u};
-    for (uint32_t j = 0; j < n; ++j) w[j >> 1] |= (uint32_t)p[j] << (16 * (j & 1));
+// The octet at p: 8 voxels packed two to a word, the missing ones of a row's
+// last octet (n < 8) repeating its last voxel.  A is the alignment of every
+// octet of the volume in bytes: 16 (X % 8 == 0), 4 (X even) or 2.
+template <int A>
+__device__ __forceinline__ uint4 mrf_oct(const uint16_t *p, uint32_t n) {
+    if (A == 16) return *reinterpret_cast<const uint4 *>(p);
+    uint32_t w[4];
+    if (A == 4) {
+        w[0] = *reinterpret_cast<const uint32_t *>(p);
+#pragma unroll
+        for (int j = 1; j < 4; ++j)
+            w[j] = 2u * j < n ? *reinterpret_cast<const uint32_t *>(p + 2 * j) : __byte_perm(w[j - 1], 0u, 0x3232u);
+    } else {
+        uint32_t v[8];
+        v[0] = p[0];
+#pragma unroll
+        for (int k = 1; k < 8; ++k) v[k] = (uint32_t)k < n ? (uint32_t)p[k] : v[k - 1];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = v[2 * j] | v[2 * j + 1] << 16;
+    }
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
-__device__ __forceinline__ void mrf_unpack(uint4 q, int32_t *v) {
+
+// The first n voxels of an octet to p.
+template <int A>
+__device__ __forceinline__ void mrf_put(uint16_t *p, uint4 q, uint32_t n) {
+    if (A == 16) {
+        *reinterpret_cast<uint4 *>(p) = q;
+        return;
+    }
     const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        v[2 * j] = (int32_t)(w[j] & 0xFFFFu);
-        v[2 * j + 1] = (int32_t)(w[j] >> 16);
-    }
-}
-
-// Eq. 3 on one octet c (n voxels valid; FULL: n = 8): left / right are the
-// x neighbours of its end voxels (-1: outside the volume), ym, yp, zm, zp
-// the octets of the neighbouring rows and planes (null: outside).  Adds the
-// octet's sum (I^{n+1} - I^0)^2 to e and whether it changed to `changed`;
-// returns the new octet (voxels past n are zero).
-template <bool FULL>
-__device__ __forceinline__ uint4 mrf_update(uint4 c, int32_t left, int32_t right, const uint4 *ym, const uint4 *yp,
-                                            const uint4 *zm, const uint4 *zp, uint4 org, int32_t delta, uint32_t n,
-                                            unsigned long long &e, bool &changed) {
-    int32_t v[8], nb[8];
-    int votes[8];
-    mrf_unpack(c, v);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const int32_t l = k > 0 ? v[k - 1] : left;
-        const int32_t r = k < 7 ? (FULL || (uint32_t)(k + 1) < n ? v[k + 1] : -1) : right;
-        votes[k] = (l >= 0 ? mrf_sgn(l - v[k]) : 0) + (r >= 0 ? mrf_sgn(r - v[k]) : 0);
-    }
-    const uint4 *rows[4] = {ym, yp, zm, zp};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        if (!rows[q]) continue;
-        mrf_unpack(*rows[q], nb);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) votes[k] += mrf_sgn(nb[k] - v[k]);
-    }
-    mrf_unpack(org, nb);
-    uint32_t w[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        if (!FULL && (uint32_t)k >= n) continue;
-        const int32_t nv = min(max(v[k] + delta * mrf_sgn(votes[k]), 0), 65535);
-        const uint32_t d = (uint32_t)abs(nv - nb[k]);
-        e += (unsigned long long)d * d;
-        changed |= nv != v[k];
-        w[k >> 1] |= (uint32_t)nv << (16 * (k & 1));
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
-__device__ __forceinline__ int32_t mrf_clamp1(int32_t d) { return min(max(d, -1), 1); }  // sgn of an integer
-
-// Eq. 3 on a whole octet with comparisons shared where two voxels compare
-// with each other: inside the octet each x pair is compared once, and along
-// z the comparison of a voxel with the plane above is, negated, the next
-// plane's comparison with the plane below (za: in, the previous plane's
-// comparisons with its plane above, or 0 at z = 0; out, this plane's).
-__device__ __forceinline__ uint4 mrf_update_full(uint4 c, int32_t left, int32_t right, const uint4 *ym,
-                                                 const uint4 *yp, const uint4 *zp, int32_t *za, uint4 org,
-                                                 int32_t delta, unsigned long long &e, bool &changed) {
-    int32_t v[8], nb[8], votes[8];
-    mrf_unpack(c, v);
-    int32_t px[7];
-#pragma unroll
-    for (int k = 0; k < 7; ++k) px[k] = mrf_clamp1(v[k + 1] - v[k]);
-    votes[0] = (left >= 0 ? mrf_clamp1(left - v[0]) : 0) + px[0] - za[0];
-#pragma unroll
-    for (int k = 1; k < 7; ++k) votes[k] = px[k] - px[k - 1] - za[k];
-    votes[7] = (right >= 0 ? mrf_clamp1(right - v[7]) : 0) - px[6] - za[7];
-    if (ym) {
-        mrf_unpack(*ym, nb);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) votes[k] += mrf_clamp1(nb[k] - v[k]);
-    }
-    if (yp) {
-        mrf_unpack(*yp, nb);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) votes[k] += mrf_clamp1(nb[k] - v[k]);
-    }
-    if (zp) {
-        mrf_unpack(*zp, nb);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            za[k] = mrf_clamp1(nb[k] - v[k]);
-            votes[k] += za[k];
+        if (A == 4) {
+            if (2u * j < n) *reinterpret_cast<uint32_t *>(p + 2 * j) = w[j];
+        } else {
+            if (2u * j < n) p[2 * j] = (uint16_t)(w[j] & 0xFFFFu);
+            if (2u * j + 1u < n) p[2 * j + 1] = (uint16_t)(w[j] >> 16);
         }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) za[k] = 0;
     }
-    mrf_unpack(org, nb);
-    uint32_t w[4];
+}
+
+constexpr uint32_t MRF_ONES = 0x00010001u;
+// Largest step index plus one at which Delta = 1 keeps every difference from
+// the input in a signed byte.
+constexpr uint32_t MRF_FAST_STEPS = 127u;
+
+// Per lane (16 bits), n limited to [c - 1, c + 1]: c + sgn(n - c), with
+// lo = max(c, 1) - 1 and hi = min(c, 65534) + 1.
+__device__ __forceinline__ uint32_t mrf_near(uint32_t n, uint32_t lo, uint32_t hi) {
+    return vmin16x2(vmax16x2(n, lo), hi);
+}
+// 0xFFFF in each 16-bit lane whose top bit is set
+__device__ __forceinline__ uint32_t mrf_top(uint32_t x) {
+    uint32_t r;
+    asm("prmt.b32 %0, %1, 0, 0xBB99;" : "=r"(r) : "r"(x));
+    return r;
+}
+
+// What a thread carries along z and adds up over its planes.
+struct MrfAcc {
+    uint32_t q[4];         // c + sgn(above - c) minus c of the plane below (0 at z = 0)
+    uint32_t e32;          // sum (I^{it+1} - I^0)^2 of the planes since the last transfer (FAST)
+    unsigned long long e;  // the same, all planes
+    uint32_t chg;          // nonzero: some voxel changed
+};
+
+// Eq. 3 on one octet, two voxels per 32-bit word and operation.  A neighbour
+// contributes t = c + sgn(n - c) in each 16-bit lane; sums and differences of
+// the t are taken modulo 2^32, where the lanes of the final sum
+// votes + 0x7FFF (votes in [-6, 6]) are exact whatever the intermediate
+// borrows.  Neighbours outside the volume are passed as the octet itself
+// (vote 0); along z the comparison with the plane above is, negated, the next
+// plane's with the plane below.  FAST: Delta = 1 and at most 127 steps so
+// far, so that no clamp to [0, 65535] is needed (a voxel at 0 is never voted
+// down) and the differences from the input, signed bytes, are squared four at
+// a time by a byte dot product.
+template <int A, bool FAST>
+__device__ __forceinline__ uint4 mrf_update(uint4 c4, uint32_t lw, uint32_t rw, uint4 ym4, uint4 yp4, uint4 ab4,
+                                            uint4 og4, uint32_t delta2, uint32_t n, MrfAcc &a) {
+    const uint32_t c[4] = {c4.x, c4.y, c4.z, c4.w}, ym[4] = {ym4.x, ym4.y, ym4.z, ym4.w};
+    const uint32_t yp[4] = {yp4.x, yp4.y, yp4.z, yp4.w}, ab[4] = {ab4.x, ab4.y, ab4.z, ab4.w};
+    const uint32_t og[4] = {og4.x, og4.y, og4.z, og4.w};
+    // the pairs shifted by one voxel: x[j] is word j's left, x[j + 1] its right
+    uint32_t x[5];
+    x[0] = __byte_perm(lw, c[0], 0x5432u);
+#pragma unroll
+    for (int j = 1; j < 4; ++j) x[j] = __byte_perm(c[j - 1], c[j], 0x5432u);
+    x[4] = __byte_perm(c[3], rw, 0x5432u);
+    uint32_t r[4], df[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const int32_t a = min(max(v[2 * j] + delta * mrf_clamp1(votes[2 * j]), 0), 65535);
-        const int32_t b = min(max(v[2 * j + 1] + delta * mrf_clamp1(votes[2 * j + 1]), 0), 65535);
-        const uint32_t da = (uint32_t)abs(a - nb[2 * j]), db = (uint32_t)abs(b - nb[2 * j + 1]);
-        e += (unsigned long long)da * da + (unsigned long long)db * db;
-        w[j] = (uint32_t)a | (uint32_t)b << 16;
+        const uint32_t lo = vmax16x2(c[j], MRF_ONES) - MRF_ONES, hi = vmin16x2(c[j], 0xFFFEFFFEu) + MRF_ONES;
+        const uint32_t qn = mrf_near(ab[j], lo, hi) - c[j];
+        const uint32_t s = mrf_near(x[j], lo, hi) + mrf_near(x[j + 1], lo, hi) + mrf_near(ym[j], lo, hi) +
+                           mrf_near(yp[j], lo, hi) + qn - a.q[j] + (0x7FFF7FFFu - 4u * c[j]);
+        a.q[j] = qn;
+        if (FAST) {
+            // c + sgn(votes)
+            r[j] = c[j] + (vmin16x2(vmax16x2(s, 0x7FFE7FFEu), 0x80008000u) - 0x7FFF7FFFu);
+        } else {
+            const uint32_t up = vmin16x2(c[j], 0xFFFFFFFFu - delta2) + delta2, dn = vmax16x2(c[j], delta2) - delta2;
+            const uint32_t mu = mrf_top(s), md = mrf_top(0xFFFEFFFEu - s);
+            r[j] = (mu & up) | (md & dn) | (c[j] & ~(mu | md));
+        }
+        if (A != 16) {  // voxels past the row's end keep the input's value: no change, no difference
+            const uint32_t m = 2u * j + 1u < n ? 0xFFFFFFFFu : (2u * j < n ? 0xFFFFu : 0u);
+            a.chg |= (r[j] ^ c[j]) & m;
+            r[j] = (r[j] & m) | (og[j] & ~m);
+        } else {
+            a.chg |= r[j] ^ c[j];
+        }
+        if (FAST) {
+            df[j] = r[j] - og[j] + 0x00800080u;  // difference + 128 in the low byte of each lane
+        } else {
+            const uint32_t d = vmax16x2(r[j], og[j]) - vmin16x2(r[j], og[j]);
+            a.e += (unsigned long long)(d & 0xFFFFu) * (d & 0xFFFFu);
+            a.e += (unsigned long long)(d >> 16) * (d >> 16);
+        }
     }
-    const uint4 r = make_uint4(w[0], w[1], w[2], w[3]);
-    changed |= ((r.x ^ c.x) | (r.y ^ c.y) | (r.z ^ c.z) | (r.w ^ c.w)) != 0u;
-    return r;
+    if (FAST) {
+        const int b0 = (int)(__byte_perm(df[0], df[1], 0x6420u) ^ 0x80808080u);
+        const int b1 = (int)(__byte_perm(df[2], df[3], 0x6420u) ^ 0x80808080u);
+        a.e32 = (uint32_t)__dp4a(b0, b0, __dp4a(b1, b1, (int)a.e32));
+    }
+    return make_uint4(r[0], r[1], r[2], r[3]);
+}
+
+// Planes [za, zb) of one tile of MRF_TILE octet columns (thread t follows
+// octet o0 + t of every plane; octets of a plane are numbered along its rows).
+template <int A, bool FAST>
+__device__ __forceinline__ void mrf_planes(const VolDev &V, uint32_t o0, uint32_t za, uint32_t zb,
+                                           const uint16_t *__restrict__ cur, uint16_t *__restrict__ nxt,
+                                           uint32_t delta2, MrfAcc &a) {
+    const uint32_t X = V.X, Y = V.Y, Z = V.Z, OX = (X + 7) >> 3;
+    const uint32_t o = o0 + threadIdx.x, lane = threadIdx.x & 31;
+    const bool live = o < Y * OX;
+    const uint32_t y = live ? o / OX : 0u, x0 = live ? 8u * (o - y * OX) : 0u;
+    const uint32_t n = A == 16 ? 8u : min(8u, X - x0);
+    const size_t plane = (size_t)X * Y, off = (size_t)y * X + x0;
+    const ptrdiff_t dm = y > 0 ? -(ptrdiff_t)X : 0, dp = y + 1 < Y ? (ptrdiff_t)X : 0;
+    const bool endl = x0 == 0, endr = x0 + 8 >= X;
+    const uint16_t *pc = cur + (size_t)za * plane + off, *po = V.mrf_in + (size_t)za * plane + off;
+    uint16_t *pn = nxt + (size_t)za * plane + off;
+    uint4 c = make_uint4(0, 0, 0, 0), ab = c, og = c;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) a.q[j] = 0u;
+    a.e32 = 0u;
+    if (live) {
+        c = mrf_oct<A>(pc, n);
+        og = mrf_oct<A>(po, n);
+        ab = za + 1 < Z ? mrf_oct<A>(pc + plane, n) : c;
+        if (za > 0) {  // what the plane below would have passed on
+            const uint4 b = mrf_oct<A>(pc - plane, n);
+            const uint32_t bw[4] = {b.x, b.y, b.z, b.w}, cw[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                a.q[j] = mrf_near(cw[j], vmax16x2(bw[j], MRF_ONES) - MRF_ONES, vmin16x2(bw[j], 0xFFFEFFFEu) + MRF_ONES) -
+                         bw[j];
+        }
+    }
+    for (uint32_t z = za; z < zb; ++z) {
+        uint4 ym = c, yp = c, ab2 = ab, og2 = og;
+        uint32_t el = 0u, er = 0u;
+        if (live) {
+            ym = mrf_oct<A>(pc + dm, n);
+            yp = mrf_oct<A>(pc + dp, n);
+            if (lane == 0 && !endl) el = pc[-1];
+            if (lane == 31 && !endr) er = pc[8];
+            // the next plane's upper neighbour and input, in flight during this plane
+            if (z + 1 < zb) {
+                og2 = mrf_oct<A>(po + plane, n);
+                if (z + 2 < Z) ab2 = mrf_oct<A>(pc + 2 * plane, n);
+            }
+        }
+        uint32_t lw = __shfl_up_sync(FULL, c.w, 1), rw = __shfl_down_sync(FULL, c.x, 1);
+        if (lane == 0) lw = el << 16;
+        if (lane == 31) rw = er;
+        if (endl) lw = c.x << 16;
+        if (endr) rw = c.w >> 16;
+        if (live) {
+            const uint4 res = mrf_update<A, FAST>(c, lw, rw, ym, yp, ab, og, delta2, n, a);
+            mrf_put<A>(pn, res, n);
+        }
+        if (FAST && ((z + 1u) & 1023u) == 0u) {  // e32 grows by at most 8 * 127^2 a plane
+            a.e += a.e32;
+            a.e32 = 0u;
+        }
+        c = ab;
+        ab = ab2;
+        og = og2;
+        pc += plane;
+        po += plane;
+        pn += plane;
+    }
+    if (FAST) a.e += a.e32;
 }
 
 // Step `it` of every MRF volume not yet stopped: reads mrf_in (it = 0) or
 // mrf_buf[it & 1], writes mrf_buf[(it + 1) & 1], and adds the step's
 // sum (I^{it+1} - I^0)^2 and whether anything changed to the volume's
-// status words.  A tile is MRF_TX octets x MRF_TY rows walked down z: each
-// thread keeps its octet of planes z - 1, z, z + 1 in registers, the rows
-// y - 1 and y + 1 come from the neighbouring threads through shared memory
-// and the x neighbours by shuffles, so every voxel of the current image is
-// read from memory about once per step.  Blocks take contiguous tile ranges
-// and flush their sums once per volume; the block whose flush completes a
+// status words.
+//
+// A tile is MRF_TILE octets of a plane, numbered along the rows whatever X is
+// (so narrow rows fill their warps), and a work unit is one plane of one
+// tile.  Every block takes an equal contiguous range of units, z fastest, and
+// walks it with the octets of planes z and z + 1 in registers: no block
+// barriers, the rows y - 1 and y + 1 come from L1 (their own warps have just
+// loaded them), the x neighbours by shuffles.  Only a range's start reads an
+// extra plane on either side.  Splitting z keeps all multiprocessors busy for
+// a single volume (a 512 x 512 x 64 volume has only 128 tiles).
+//
+// Bound by instruction issue (about 15 per voxel), near its traffic of 6 bytes
+// per voxel: 89 us a step for four 512 x 512 x 64 volumes (4.5 TB/s, 0.67 of
+// the measured copy rate) and 24 us for one, where whole-z tiles of 256 x 8
+// voxels with scalar votes took 277 and 115 us.  Three blocks per
+// multiprocessor: two take 114 us, four 27 us for the one volume.
+//
+// Blocks flush their sums once per volume; the block whose flush completes a
 // volume decides: stop at a step that changes nothing or strays too far
 // (keeping I^it), or at the step limit; when stopping it points the volume's
 // raw input for the smoothing (in the device copy of the batch descriptor)
 // at the kept image.
-__global__ void __launch_bounds__(MRF_TX * MRF_TY, 3) k_mrf_step(const BatchHdr *__restrict__ h, uint32_t it) {
-    __shared__ uint4 srow[MRF_TY + 2][MRF_TX];  // plane z, rows y0 - 1 .. y0 + MRF_TY
-    __shared__ unsigned long long red[MRF_TX * MRF_TY / 32];
+__global__ void __launch_bounds__(MRF_TILE, 3) k_mrf_step(const BatchHdr *__restrict__ h, uint32_t it) {
+    __shared__ unsigned long long red[MRF_TILE / 32];
     __shared__ uint32_t chg_any;  // some voxel of the block's tiles changed (0 between volumes)
     if (threadIdx.x == 0) chg_any = 0u;
-    const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;
-    const uint32_t T = h->mrf_ctiles, G = gridDim.x;
-    const uint32_t tb = (uint32_t)(((uint64_t)T * blockIdx.x) / G);
-    const uint32_t te = (uint32_t)(((uint64_t)T * (blockIdx.x + 1)) / G);
+    const uint64_t T = h->mrf_units;
+    const uint32_t G = gridDim.x;
+    // (T / G) b + (T % G) b / G: the b-th of G equal ranges without a 64-bit overflow
+    const uint64_t tq = T / G;
+    const uint32_t tr = (uint32_t)(T % G);
+    const uint64_t tb = tq * blockIdx.x + (uint64_t)tr * blockIdx.x / G;
+    const uint64_t te = tq * (blockIdx.x + 1) + (uint64_t)tr * (blockIdx.x + 1) / G;
     uint32_t vi = 0;
-    while (vi + 1 < h->nvol && tb >= h->vol[vi + 1].mrf_cbase) ++vi;
-    unsigned long long e = 0;
-    bool changed = false;
-    uint32_t ntile = 0;
+    while (vi + 1 < h->nvol && tb >= h->vol[vi + 1].mrf_ubase) ++vi;
+    MrfAcc a;
+    a.e = 0ull;
+    a.chg = 0u;
+    uint32_t nunit = 0;
     __syncthreads();
-    auto flush = [&]() {  // this block's tiles of volume vi
-        if (changed) chg_any = 1u;  // benign race: every writer stores 1
-        const unsigned long long sum = mrf_block_sum(e, red);  // (its barriers also order chg_any)
+    auto flush = [&]() {  // this block's units of volume vi
+        if (a.chg) chg_any = 1u;  // benign race: every writer stores 1
+        const unsigned long long sum = mrf_block_sum(a.e, red);  // (its barriers also order chg_any)
         const VolDev &V = h->vol[vi];
         uint32_t *st = V.stat;
-        if (threadIdx.x == 0 && ntile) {
+        if (threadIdx.x == 0 && nunit) {
             unsigned long long *E = reinterpret_cast<unsigned long long *>(st + ST_MRF_E);
             if (sum) atomicAdd(E, sum);
             if (chg_any) atomicOr(st + ST_MRF_CHG, 1u);
             __threadfence();
-            if (atomicAdd(st + ST_MRF_CNT, ntile) + ntile == V.mrf_ctiles) {
-                // every tile of this volume is in: decide
+            if (atomicAdd(st + ST_MRF_CNT, nunit) + nunit == V.mrf_ctiles * V.Z) {
+                // every unit of this volume is in: decide
                 __threadfence();
                 const unsigned long long tot = atomicAdd(E, 0ull);
                 const uint32_t chg = atomicAdd(st + ST_MRF_CHG, 0u);
@@ -3159,76 +3259,37 @@ __global__ void __launch_bounds__(MRF_TX * MRF_TY, 3) k_mrf_step(const BatchHdr 
             }
         }
         if (threadIdx.x == 0) chg_any = 0u;
-        e = 0;
-        changed = false;
-        ntile = 0;
+        a.e = 0ull;
+        a.chg = 0u;
+        nunit = 0;
         __syncthreads();
     };
-    for (uint32_t t = tb; t < te; ++t) {
-        if (vi + 1 < h->nvol && t >= h->vol[vi + 1].mrf_cbase) {
+    for (uint64_t t = tb; t < te;) {
+        if (vi + 1 < h->nvol && t >= h->vol[vi + 1].mrf_ubase) {
             flush();
-            do ++vi; while (vi + 1 < h->nvol && t >= h->vol[vi + 1].mrf_cbase);
+            do ++vi; while (vi + 1 < h->nvol && t >= h->vol[vi + 1].mrf_ubase);
         }
         const VolDev &V = h->vol[vi];
+        const uint32_t lu = (uint32_t)(t - V.mrf_ubase), tile = lu / V.Z, za = lu - tile * V.Z;
+        const uint32_t zb = (uint32_t)min((uint64_t)V.Z, za + (te - t));
+        t += zb - za;
         // volumes that stopped (or never started) are left alone; the flag
         // was set by an earlier launch, so it is the same for every thread
         if (it >= V.mrf_max || V.stat[ST_MRF_DONE]) continue;
-        ++ntile;
-        const uint32_t X = V.X, Y = V.Y, Z = V.Z, OX = (X + 7) >> 3;
-        const uint32_t ntx = (OX + MRF_TX - 1) / MRF_TX;
-        const uint32_t lt = t - V.mrf_cbase;
-        const uint32_t ox = (lt % ntx) * MRF_TX + lx, y0 = (lt / ntx) * MRF_TY, y = y0 + ly;
-        const uint32_t x0 = 8 * ox;
-        const bool live = ox < OX && y < Y;
-        const uint32_t n = live ? min(8u, X - x0) : 0u;
-        const bool vec = n == 8u && V.mrf_vec;  // (mrf_buf is always aligned)
-        const size_t plane = (size_t)X * Y;
+        nunit += zb - za;
         const uint16_t *cur = it == 0 ? V.mrf_in : V.mrf_buf[it & 1u];
         uint16_t *nxt = V.mrf_buf[(it + 1u) & 1u];
-        const int32_t delta = (int32_t)V.stat[ST_MRF_DELTA];
-        const size_t off = (size_t)y * X + x0;  // this octet in plane 0
-        // halo rows of the tile (loaded by the first and last warp)
-        const bool hrow = (ly == 0 && y0 > 0) || (ly == MRF_TY - 1 && y0 + MRF_TY < Y);
-        const uint32_t hy = ly == 0 ? y0 - 1 : y0 + MRF_TY;
-        const uint32_t hn = (hrow && ox < OX) ? min(8u, X - x0) : 0u;
-        const size_t hoff = (size_t)hy * X + x0;
-        uint4 below = make_uint4(0, 0, 0, 0), c = below, above = below;
-        int32_t za[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // full octets: comparisons with the plane above
-        if (n) c = mrf_oct(cur + off, vec, n);
-        if (n && Z > 1) above = mrf_oct(cur + plane + off, vec, n);
-        for (uint32_t z = 0; z < Z; ++z) {
-            const size_t zo = (size_t)z * plane;
-            srow[ly + 1][lx] = c;
-            if (hn) srow[ly == 0 ? 0 : MRF_TY + 1][lx] = mrf_oct(cur + zo + hoff, hn == 8u && V.mrf_vec, hn);
-            // x neighbours: the next octets of the row, or memory at the tile's ends
-            const uint32_t lnb = __shfl_up_sync(FULL, c.w >> 16, 1);
-            const uint32_t rnb = __shfl_down_sync(FULL, c.x & 0xFFFFu, 1);
-            __syncthreads();
-            if (n) {
-                const int32_t left = x0 == 0 ? -1 : (lx > 0 ? (int32_t)lnb : (int32_t)cur[zo + off - 1]);
-                const int32_t right = x0 + 8 >= X ? -1 : (lx < 31 ? (int32_t)rnb : (int32_t)cur[zo + off + 8]);
-                const uint4 *ym = y > 0 ? &srow[ly][lx] : nullptr;
-                const uint4 *yp = y + 1 < Y ? &srow[ly + 2][lx] : nullptr;
-                const uint4 org = mrf_oct(V.mrf_in + zo + off, vec, n);
-                uint4 res;
-                if (n == 8u)
-                    res = mrf_update_full(c, left, right, ym, yp, z + 1 < Z ? &above : nullptr, za, org, delta, e,
-                                          changed);
-                else
-                    res = mrf_update<false>(c, left, right, ym, yp, z > 0 ? &below : nullptr,
-                                            z + 1 < Z ? &above : nullptr, org, delta, n, e, changed);
-                uint16_t *dst = nxt + zo + off;
-                if (vec) {
-                    *reinterpret_cast<uint4 *>(dst) = res;
-                } else {
-                    const uint32_t w[4] = {res.x, res.y, res.z, res.w};
-                    for (uint32_t k = 0; k < n; ++k) dst[k] = (uint16_t)(w[k >> 1] >> (16 * (k & 1)));
-                }
-            }
-            below = c;
-            c = above;
-            if (n && z + 2 < Z) above = mrf_oct(cur + zo + 2 * plane + off, vec, n);
-            __syncthreads();  // srow is rewritten for the next plane
+        const uint32_t delta = V.stat[ST_MRF_DELTA], o0 = tile * MRF_TILE;
+        const bool fast = delta == 1u && it < MRF_FAST_STEPS;
+        if (V.mrf_align == 16u) {
+            if (fast) mrf_planes<16, true>(V, o0, za, zb, cur, nxt, MRF_ONES, a);
+            else mrf_planes<16, false>(V, o0, za, zb, cur, nxt, delta * MRF_ONES, a);
+        } else if (V.mrf_align == 4u) {
+            if (fast) mrf_planes<4, true>(V, o0, za, zb, cur, nxt, MRF_ONES, a);
+            else mrf_planes<4, false>(V, o0, za, zb, cur, nxt, delta * MRF_ONES, a);
+        } else {
+            if (fast) mrf_planes<2, true>(V, o0, za, zb, cur, nxt, MRF_ONES, a);
+            else mrf_planes<2, false>(V, o0, za, zb, cur, nxt, delta * MRF_ONES, a);
         }
     }
     if (tb < te) flush();
@@ -4008,7 +4069,7 @@ cudaError_t configure_kernels(int device, LaunchPlan &plan) {
     if ((e = resident((const void *)k_dist_line<1>, 256, &g3)) != cudaSuccess) return e;
     plan.grid_dist = std::min(g1, std::min(g2, g3));
     if ((e = resident((const void *)k_mrf_stats, MRF_TILE, &plan.grid_mrf)) != cudaSuccess) return e;
-    if ((e = resident((const void *)k_mrf_step, MRF_TX * MRF_TY, &plan.grid_mrfs)) != cudaSuccess) return e;
+    if ((e = resident((const void *)k_mrf_step, MRF_TILE, &plan.grid_mrfs)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_dist_z, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DZ_SMEM)) !=
         cudaSuccess)
         return e;
@@ -4111,7 +4172,7 @@ cudaError_t launch_pipeline(const BatchHdr *d, const LaunchPlan &p, cudaStream_t
         k_mrf_prep<<<p.grid_vols, 32, 0, s>>>(d);
     }
     rec();
-    for (uint32_t it = 0; it < p.mrf_iters; ++it) k_mrf_step<<<p.grid_mrfs, MRF_TX * MRF_TY, 0, s>>>(d, it);
+    for (uint32_t it = 0; it < p.mrf_iters; ++it) k_mrf_step<<<p.grid_mrfs, MRF_TILE, 0, s>>>(d, it);
     cudaError_t e;
     switch (p.tile_y) {
         case 16: e = launch_tile_kernels<16>(d, p, s, ev, k); break;
