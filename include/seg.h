@@ -222,8 +222,8 @@ int seg_read_labels(seg_ctx *ctx, seg_req req, uint32_t channel, uint32_t *dst,
  * into a zeroed X*Y*Z image gives exactly seg_read_labels' image; a row of
  * X voxels holds at most ceil(X/2) runs.  *n_runs gets the number of runs.
  * dst holds cap runs in host memory, or device memory when dst_on_device = 1;
- * dst = NULL with cap = 0 only reports the number.  Derived on the device
- * from the label image (two passes over it) and copied; blocks until done.
+ * dst = NULL with cap = 0 only reports the number.  Taken from the run records
+ * kept with the cells (or, where they found no room, from the label image); blocks until done.
  * Errors: SEG_ESMALL (cap < *n_runs, nothing written); SEG_ETOOBIG for an
  * image of more than 2^32 - 65 rows; otherwise as seg_read_labels. */
 int seg_read_label_runs(seg_ctx *ctx, seg_req req, uint32_t channel, seg_label_run *dst, uint64_t cap,

@@ -16,7 +16,7 @@ enum StatWord : uint32_t {
     ST_THRESH = 0,     // Otsu level t* (foreground = s > t*)
     ST_RUNS = 1,       // number of foreground runs R
     ST_CELLS = 2,      // number of surviving cells K
-    // word 3 unused
+    ST_LABEL_RUNS = 3, // number of runs of surviving cells
     ST_ERROR = 4,      // error bits (ERR_*)
     ST_MRF_STEPS = 5,  // MRF denoise: steps kept
     ST_MRF_SEL = 6,    // MRF denoise: result buffer (0 input, 1 mrf_buf[0], 2 mrf_buf[1])
@@ -223,6 +223,33 @@ cudaError_t launch_denoise(const BatchHdr *d_hdr, const LaunchPlan &plan, cudaSt
 // Cell-to-vessel distance: out[k - 1] = min of map over the voxels labelled k.
 cudaError_t launch_cell_distance(const uint32_t *labels, const uint32_t *map, uint64_t n, uint32_t *out, uint64_t k,
                                  int sms, cudaStream_t s);
+// Where k_label_features leaves a volume's run records: at the end of its
+// cell table (k_cap cells of 64 bytes, of which the first K are used), when
+// they fit there behind the K cells.  words: R records of three words (the
+// fields of a seg_label_run, label 0 for a dropped run); tiles: per row tile
+// its first run and its number of labelled runs.  Null: no room.
+struct RunRecords {
+    uint32_t *words;
+    uint2 *tiles;
+    __host__ __device__ RunRecords(seg_cell_features *feat, uint64_t k_cap, uint32_t cells, uint32_t runs,
+                                   uint32_t nrt) {
+        const uint64_t room = sizeof(seg_cell_features) * k_cap, used = sizeof(seg_cell_features) * (uint64_t)cells;
+        const uint64_t table = 8ull * nrt, need = table + 12ull * runs;
+        words = nullptr;
+        tiles = nullptr;
+        if (used + need > room) return;
+        char *at = reinterpret_cast<char *>(feat) + ((room - need) & ~15ull);
+        if (at < reinterpret_cast<char *>(feat) + used) return;
+        tiles = reinterpret_cast<uint2 *>(at);
+        words = reinterpret_cast<uint32_t *>(at + table);
+    }
+};
+
+// The labelled runs of the records, in order, as three words each into out
+// (device memory or mapped host memory).
+cudaError_t launch_runs_compact(const RunRecords &rec, uint32_t ntiles, uint32_t runs, uint32_t *out, int sms,
+                                cudaStream_t s);
+
 // Label runs of one label image (rows = Y*Z rows of X voxels): the count
 // pass (per-row counts into rowcnt, per-block offsets into tiles, the total
 // into *total) and the write pass (records into out, nothing when *total >

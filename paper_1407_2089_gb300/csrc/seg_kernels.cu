@@ -2141,6 +2141,13 @@ __device__ __forceinline__ void feat_global(seg_cell_features *f, unsigned long 
 // folds the run's contribution to its cell (count, coordinate sums, bounding
 // box) into a shared table; after a barrier the table goes to the global
 // cells with one set of atomics per (tile, cell).
+//
+// The same loop writes every run as a seg_label_run (label 0: its component
+// was dropped) for seg_read_label_runs, into the part of the cell table that
+// no cell uses (RunRecords: the table is sized for the most cells the volume
+// can hold), with the tile's first run and number of labelled runs.  Reading
+// the runs then moves the records (0.7 MB for a 512 x 512 x 64 frame) and not
+// the label image twice (134 MB).
 constexpr int LABEL_RUNS = 2048;
 
 __global__ void __launch_bounds__(ROW_TILE, 6) k_label_features(const BatchHdr *__restrict__ h) {
@@ -2152,12 +2159,14 @@ __global__ void __launch_bounds__(ROW_TILE, 6) k_label_features(const BatchHdr *
     __shared__ uint2 srl[LABEL_RUNS];  // staged runs: x0 | x1 << 16, final label
     __shared__ uint8_t srow[LABEL_RUNS];  // row of each staged run in the tile
     __shared__ FeatTable T;
+    __shared__ uint32_t skept;  // labelled runs of the tile
     for (uint32_t rt = blockIdx.x; rt < h->nrowtiles; rt += gridDim.x) {
         const VolDev &V = h->vol[VI.find(h, rt)];
         const uint32_t lt = rt - V.rt_base;
         const uint32_t row0 = lt * h->row_tile;
         const uint32_t nrows = min(h->row_tile, V.rows - row0);
         __syncthreads();  // previous tile done with soff, srl and T
+        if (tid == 0) skept = 0u;
         for (uint32_t i = tid; i <= nrows; i += ROW_TILE) soff[i] = V.rowoff[row0 + i];
         T.key[tid] = 0u;
         T.cx[tid] = T.sy[tid] = T.sz[tid] = 0ull;
@@ -2266,9 +2275,11 @@ __global__ void __launch_bounds__(ROW_TILE, 6) k_label_features(const BatchHdr *
                 }
             }
         }
+        const RunRecords rec(V.feat, V.k_cap, V.stat[ST_CELLS], V.stat[ST_RUNS], V.nrt);
+        uint32_t kept = 0;
         for (uint32_t j = rb + tid; j < re; j += ROW_TILE) {
             const uint32_t lab = run_label(j);
-            if (!lab || lab > V.k_cap) continue;
+            kept += lab != 0u;
             uint32_t lo;
             if (staged) {
                 lo = srow[j - rb];
@@ -2282,8 +2293,15 @@ __global__ void __launch_bounds__(ROW_TILE, 6) k_label_features(const BatchHdr *
                 }
             }
             const uint32_t row = row0 + lo;
-            const uint32_t y = row % V.Y, z = row / V.Y;
             const uint32_t rx = run_x(j);
+            if (rec.words) {
+                uint32_t *o = rec.words + 3ull * j;
+                o[0] = lab;
+                o[1] = row;
+                o[2] = rx;
+            }
+            if (!lab || lab > V.k_cap) continue;
+            const uint32_t y = row % V.Y, z = row / V.Y;
             const uint32_t x0 = rx & 0xFFFFu, x1 = rx >> 16;
             const unsigned long long len = x1 - x0 + 1u;
             const unsigned long long sx = ((unsigned long long)(x0 + x1) * len) >> 1;
@@ -2310,7 +2328,13 @@ __global__ void __launch_bounds__(ROW_TILE, 6) k_label_features(const BatchHdr *
                 feat_global(V.feat + (lab - 1), len, sx, len * y, len * z, mn, mx);
             }
         }
+        kept = __reduce_add_sync(FULL, kept);
+        if (lane == 0 && kept) atomicAdd(&skept, kept);
         __syncthreads();
+        if (tid == 0) {
+            if (rec.words) rec.tiles[lt] = make_uint2(rb, skept);
+            if (skept) atomicAdd(V.stat + ST_LABEL_RUNS, skept);
+        }
         {
             const uint32_t lab = T.key[tid];
             if (lab) {
@@ -3876,7 +3900,45 @@ __global__ void __launch_bounds__(256) k_cell_distance(const uint32_t *__restric
     }
 }
 
-// Label runs (read path; Segmentation section: each cell's voxels, the set
+// Label runs from the records k_label_features left (rows in order, label 0
+// for dropped runs): the labelled ones, in order.  One block per row tile at a
+// time: its runs start at the sum of the tiles' labelled runs below it, 256
+// records at a time are ranked by a block scan, gathered in shared memory and
+// written as consecutive words.
+__global__ void __launch_bounds__(ROW_TILE) k_runs_compact(const uint32_t *__restrict__ rec,
+                                                           const uint2 *__restrict__ tiles, uint32_t ntiles,
+                                                           uint32_t runs, uint32_t *__restrict__ out) {
+    __shared__ uint32_t sbuf[33];
+    __shared__ uint32_t stage[3 * ROW_TILE];
+    const uint32_t tid = threadIdx.x;
+    for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        const uint32_t rb = tiles[t].x, re = t + 1 < ntiles ? tiles[t + 1].x : runs;
+        uint32_t below = 0;
+        for (uint32_t i = tid; i < t; i += ROW_TILE) below += tiles[i].y;
+        uint64_t at = block_sum<ROW_TILE>(below, sbuf);
+        for (uint32_t j0 = rb; j0 < re; j0 += ROW_TILE) {
+            const uint32_t j = j0 + tid;
+            uint32_t w[3] = {0u, 0u, 0u};
+            if (j < re) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) w[k] = rec[3ull * j + k];
+            }
+            uint32_t n;
+            const uint32_t r = block_exscan<ROW_TILE>(w[0] != 0u, &n, sbuf);
+            if (w[0]) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) stage[3u * r + k] = w[k];
+            }
+            __syncthreads();
+            for (uint32_t i = tid; i < 3u * n; i += ROW_TILE) out[3ull * at + i] = stage[i];
+            at += n;
+            __syncthreads();  // stage and sbuf are reused
+        }
+    }
+}
+
+// Label runs from the label image, for volumes whose cell table has no room
+// for the run records (Segmentation section: each cell's voxels, the set
 // handed to the convex hull step): the maximal runs of equal non-zero label
 // along x, in order of (row, x).  With L = 0 outside the row, a run starts at
 // x when L(x) != 0 and L(x) != L(x - 1), and ends at x - 1 when L(x - 1) != 0
@@ -4115,6 +4177,13 @@ cudaError_t launch_cell_distance(const uint32_t *labels, const uint32_t *map, ui
     const uint64_t want = (n + 8 * 256 - 1) / (8 * 256);
     const int grid = (int)std::min<uint64_t>(want, (uint64_t)sms * 8);
     k_cell_distance<<<grid, 256, 0, s>>>(labels, map, n, k, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_runs_compact(const RunRecords &rec, uint32_t ntiles, uint32_t runs, uint32_t *out, int sms,
+                                cudaStream_t s) {
+    const int grid = (int)std::min<uint64_t>(ntiles, (uint64_t)sms * 8);
+    k_runs_compact<<<grid, ROW_TILE, 0, s>>>(rec.words, rec.tiles, ntiles, runs, out);
     return cudaGetLastError();
 }
 

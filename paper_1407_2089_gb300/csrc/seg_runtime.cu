@@ -123,6 +123,7 @@ struct Request {
     std::vector<size_t> off_den;          // per channel; SIZE_MAX = no denoise (front end: 1 image, MRF: 2)
     size_t off_smooth = SIZE_MAX;         // smoothed images of all channels (SEG_KEEP_SMOOTHED)
     std::vector<uint32_t> mrf_steps, mrf_sel;
+    std::vector<uint32_t> runs, label_runs, nrt;  // foreground runs, runs of the cells, row tiles of the batch
     size_t per_labels = 0, per_feat = 0;  // bytes per channel
     bool owns_input = false;
     bool admitted = false;
@@ -204,7 +205,6 @@ struct seg_ctx {
     bool tuned = false;  // tile shape fixed (forced, or tuned on the first batch)
     cudaStream_t copy_stream = nullptr;
     cudaStream_t read_stream = nullptr;
-    uint32_t *read_pin = nullptr;  // pinned words for small results of the read calls (one reader at a time)
     std::vector<Slot> slots;
     std::mutex mu;
     std::condition_variable cv;
@@ -681,6 +681,9 @@ void finalize_batch(seg_ctx *ctx, Slot &s) {
             r->errbits[c] = w[ST_ERROR];
             r->mrf_steps[c] = w[ST_MRF_STEPS];
             r->mrf_sel[c] = w[ST_MRF_SEL];
+            r->runs[c] = w[ST_RUNS];
+            r->label_runs[c] = w[ST_LABEL_RUNS];
+            r->nrt[c] = s.h_hdr->vol[v].nrt;
             if (w[ST_ERROR]) bad = true;
         }
         r->state = bad ? SEG_FAILED : SEG_DONE;
@@ -901,7 +904,6 @@ int seg_create(const seg_config *cfg, seg_ctx **out) {
     cudaGetLastError();
     CK(cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking));
     CK(cudaStreamCreateWithFlags(&ctx->read_stream, cudaStreamNonBlocking));
-    CK(cudaMallocHost(reinterpret_cast<void **>(&ctx->read_pin), 64));
     ctx->slots.resize(nslots);
     for (Slot &s : ctx->slots) {
         CK(cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking));
@@ -945,7 +947,6 @@ int seg_destroy(seg_ctx *ctx) {
     }
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     if (ctx->read_stream) cudaStreamDestroy(ctx->read_stream);
-    if (ctx->read_pin) cudaFreeHost(ctx->read_pin);
     delete ctx;
     return SEG_OK;
 }
@@ -1002,6 +1003,9 @@ int seg_submit_volume(seg_ctx *ctx, const uint16_t *voxels, int on_device, seg_d
     r->ncells.assign(channels, 0);
     r->mrf_steps.assign(channels, 0);
     r->mrf_sel.assign(channels, 0);
+    r->runs.assign(channels, 0);
+    r->label_runs.assign(channels, 0);
+    r->nrt.assign(channels, 0);
     r->errbits.assign(channels, 0);
     r->owns_input = host_in;
     if (!host_in) r->user_dev = voxels;
@@ -1237,64 +1241,66 @@ int seg_read_label_runs(seg_ctx *ctx, seg_req req, uint32_t channel, seg_label_r
     if (channel >= r->C || (!dst && cap)) return SEG_EINVAL;
     const VolGeom &g = r->g[channel];
     if (g.rows > 0xFFFFFFFFu - 64u) return SEG_ETOOBIG;  // row indices of the blocks stay in 32 bits
-    const uint32_t nt = label_runs_tiles(g.rows);
-    const size_t a_rows = al(4ull * g.rows), a_tiles = al(4ull * nt);
-    const uint64_t most = (uint64_t)g.rows * ((g.X + 1) / 2);  // runs a label image can hold
+    const uint32_t total = r->label_runs[channel];
+    if (n_runs) *n_runs = total;
+    if (cap < total) return dst ? SEG_ESMALL : SEG_OK;
+    if (!dst || !total) return SEG_OK;
     cudaSetDevice(ctx->device);
     cudaStream_t s = ctx->read_stream;
-    // A destination the device reaches (device memory, or pinned host
-    // memory through its mapping) takes the records in the same pass of
-    // launches as the count, with one synchronisation; pageable memory is
-    // filled by a copy once the count is known.
-    seg_label_run *mapped = nullptr;
-    if (dst && cap && !dst_on_device) {
+    const size_t bytes = sizeof(seg_label_run) * (size_t)total;
+    const RunRecords rec(r->feat(channel), g.k_cap, r->ncells[channel], r->runs[channel], r->nrt[channel]);
+    if (rec.words && total == r->runs[channel]) {
+        // every run is labelled: the records are the result
+        cudaError_t e = cudaMemcpyAsync(dst, rec.words, bytes,
+                                        dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        return cuda_fail(e, "seg_read_label_runs");
+    }
+    // A destination the device reaches (device memory, or pinned host memory
+    // through its mapping) is written by the kernels; pageable memory is
+    // filled by a copy.
+    seg_label_run *direct = dst_on_device ? dst : nullptr, *mapped = nullptr;
+    if (!dst_on_device) {
         cudaPointerAttributes pa;
         if (cudaPointerGetAttributes(&pa, dst) == cudaSuccess && pa.type == cudaMemoryTypeHost && pa.devicePointer)
             mapped = static_cast<seg_label_run *>(pa.devicePointer);
         cudaGetLastError();
     }
-    const bool one_pass = dst && cap && (dst_on_device || mapped);
-    const uint64_t stage = mapped ? std::min<uint64_t>(cap, most) : 0;
+    seg_label_run *out = direct, *stage = nullptr;
     char *tmp = nullptr;
-    seg_label_run *dev_out = nullptr;
-    uint32_t total = 0;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&tmp), a_rows + a_tiles + 256, s);
-    uint32_t *rowcnt = reinterpret_cast<uint32_t *>(tmp);
-    uint32_t *tiles = reinterpret_cast<uint32_t *>(tmp + a_rows);
-    uint32_t *d_total = reinterpret_cast<uint32_t *>(tmp + a_rows + a_tiles);
-    if (e == cudaSuccess) e = launch_label_runs_count(r->labels(channel), g.X, g.rows, rowcnt, tiles, d_total,
-                                                      ctx->sms, s);
-    if (one_pass) {
-        dev_out = dst_on_device ? dst : nullptr;
-        if (e == cudaSuccess && mapped && stage)
-            e = cudaMallocAsync(reinterpret_cast<void **>(&dev_out), sizeof(seg_label_run) * stage, s);
-        if (e == cudaSuccess && dev_out)
-            e = launch_label_runs_write(r->labels(channel), g.X, g.rows, rowcnt, tiles, d_total,
-                                        mapped ? stage : cap, dev_out, mapped, ctx->sms, s);
-        if (mapped && dev_out) cudaFreeAsync(dev_out, s);
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->read_pin, d_total, 4, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    int rc = SEG_OK;
-    if (e == cudaSuccess) {
-        total = ctx->read_pin[0];
-        if (n_runs) *n_runs = total;
-        if (cap < total) {
-            rc = dst ? SEG_ESMALL : SEG_OK;
-        } else if (total && !one_pass) {
-            e = cudaMallocAsync(reinterpret_cast<void **>(&dev_out), sizeof(seg_label_run) * total, s);
-            if (e == cudaSuccess)
-                e = launch_label_runs_write(r->labels(channel), g.X, g.rows, rowcnt, tiles, d_total, total, dev_out,
-                                            nullptr, ctx->sms, s);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(dst, dev_out, sizeof(seg_label_run) * total, cudaMemcpyDeviceToHost, s);
-            if (dev_out) cudaFreeAsync(dev_out, s);
+    cudaError_t e = cudaSuccess;
+    if (rec.words) {
+        if (mapped) out = mapped;
+        if (!out) {
+            e = cudaMallocAsync(reinterpret_cast<void **>(&stage), bytes, s);
+            out = stage;
         }
+        if (e == cudaSuccess)
+            e = launch_runs_compact(rec, r->nrt[channel], r->runs[channel], reinterpret_cast<uint32_t *>(out),
+                                    ctx->sms, s);
+    } else {
+        // no room for the records: two passes over the label image
+        const uint32_t nt = label_runs_tiles(g.rows);
+        const size_t a_rows = al(4ull * g.rows), a_tiles = al(4ull * nt);
+        e = cudaMallocAsync(reinterpret_cast<void **>(&tmp), a_rows + a_tiles + 256, s);
+        uint32_t *rowcnt = reinterpret_cast<uint32_t *>(tmp);
+        uint32_t *tiles = reinterpret_cast<uint32_t *>(tmp + a_rows);
+        uint32_t *d_total = reinterpret_cast<uint32_t *>(tmp + a_rows + a_tiles);
+        if (e == cudaSuccess)
+            e = launch_label_runs_count(r->labels(channel), g.X, g.rows, rowcnt, tiles, d_total, ctx->sms, s);
+        if (e == cudaSuccess && !out) {
+            e = cudaMallocAsync(reinterpret_cast<void **>(&stage), bytes, s);
+            out = stage;
+        }
+        if (e == cudaSuccess)
+            e = launch_label_runs_write(r->labels(channel), g.X, g.rows, rowcnt, tiles, d_total, total, out, mapped,
+                                        ctx->sms, s);
     }
+    if (e == cudaSuccess && stage && !mapped) e = cudaMemcpyAsync(dst, stage, bytes, cudaMemcpyDeviceToHost, s);
+    if (stage) cudaFreeAsync(stage, s);
     if (tmp) cudaFreeAsync(tmp, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(e, "seg_read_label_runs");
-    return rc;
+    const cudaError_t es = cudaStreamSynchronize(s);
+    return cuda_fail(e == cudaSuccess ? es : e, "seg_read_label_runs");
 }
 
 int seg_read_distance(seg_ctx *ctx, seg_req req, uint32_t channel, uint32_t *dst, uint64_t dst_elems,
