@@ -41,6 +41,10 @@ constexpr int TILE_X = 64;        // smoothing tile width (outputs along x)
 constexpr uint32_t UNION_LIMIT = 1u << 24;  // union-find retries before ERR_UNION
 constexpr int ROW_TILE = 256;     // rows per row tile (run kernels; their block size)
 constexpr int ROW_TILE_MIN = 32;  // smallest row tile (batches with few rows)
+// Label tile: LABEL_WORDS label words (256 KB) in whole rows, at most ROW_TILE
+// rows; halved for batches with few tiles, down to LABEL_WORDS >> LABEL_SHRINK.
+constexpr uint32_t LABEL_WORDS = 65536;
+constexpr uint32_t LABEL_SHRINK = 4;
 constexpr int HIST_BINS = 65536;
 // Union-find bricks: BRICK_Y x BRICK_Z rows (one thread each) whose runs are
 // united in shared memory when there are at most BRICK_CAP of them.
@@ -85,6 +89,9 @@ struct VolDev {
     uint32_t fs_ntx, fs_nty, fs_ntz;  // tiles per axis
     uint32_t fs_base;         // first flat k_smooth_rows tile index
     uint32_t rt_base;         // first flat row-tile index
+    uint32_t lb_rows;         // rows per label tile (at most ROW_TILE)
+    uint32_t nlb;             // label tiles
+    uint32_t lb_base;         // first flat label-tile index
     uint32_t nby;             // union-find bricks along y
     uint32_t nbk;             // union-find bricks
     uint32_t bk_base;         // first flat brick index
@@ -163,6 +170,7 @@ struct BatchHdr {
     uint64_t mrf_units;       // k_mrf_step units over the batch
     uint32_t row_tile;        // rows per row tile: ROW_TILE, or down to ROW_TILE_MIN
                               // so that a batch with few rows still fills the GPU
+    uint32_t nlabtiles;       // label tiles over the batch
     VolDev vol[1];       // nvol entries
 };
 
@@ -226,15 +234,15 @@ cudaError_t launch_cell_distance(const uint32_t *labels, const uint32_t *map, ui
 // Where k_label_features leaves a volume's run records: at the end of its
 // cell table (k_cap cells of 64 bytes, of which the first K are used), when
 // they fit there behind the K cells.  words: R records of three words (the
-// fields of a seg_label_run, label 0 for a dropped run); tiles: per row tile
-// its first run and its number of labelled runs.  Null: no room.
+// fields of a seg_label_run, label 0 for a dropped run); tiles: per
+// label tile its first run and its number of labelled runs.  Null: no room.
 struct RunRecords {
     uint32_t *words;
     uint2 *tiles;
     __host__ __device__ RunRecords(seg_cell_features *feat, uint64_t k_cap, uint32_t cells, uint32_t runs,
-                                   uint32_t nrt) {
+                                   uint32_t ntiles) {
         const uint64_t room = sizeof(seg_cell_features) * k_cap, used = sizeof(seg_cell_features) * (uint64_t)cells;
-        const uint64_t table = 8ull * nrt, need = table + 12ull * runs;
+        const uint64_t table = 8ull * ntiles, need = table + 12ull * runs;
         words = nullptr;
         tiles = nullptr;
         if (used + need > room) return;

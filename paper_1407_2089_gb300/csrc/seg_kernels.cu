@@ -2097,16 +2097,26 @@ __global__ void __launch_bounds__(ROW_TILE) k_rank(const BatchHdr *__restrict__ 
 constexpr int FEAT_SLOTS = 256;
 constexpr int FEAT_PROBES = 8;
 
-// cx packs a cell's voxel count in a row tile (at most 256 * 65536 = 2^24,
-// 25 bits) under its x-coordinate sum (at most 256 * (0 + ... + 65535) < 2^39),
-// so one 64-bit add carries both exactly.
-constexpr int CX_SHIFT = 25;
-
+// Sums are kept as 32-bit words (a 64-bit shared add is a compare-and-swap
+// loop, and neighbouring runs of one cell collide in it: with 64-bit sums the
+// label kernel took 50 us more of 400 on 32 time-lapse channels).
 struct FeatTable {
     uint32_t key[FEAT_SLOTS];
-    unsigned long long cx[FEAT_SLOTS], sy[FEAT_SLOTS], sz[FEAT_SLOTS];
+    uint32_t cnt[FEAT_SLOTS];  // at most 256 * 65536
+    uint32_t lo[3][FEAT_SLOTS], hi[3][FEAT_SLOTS];
     uint32_t mn[3][FEAT_SLOTS], mx[3][FEAT_SLOTS];
 };
+
+// Adds v to the sum hi : lo.  narrow: no sum of the tile reaches 2^32.
+__device__ __forceinline__ void sadd(uint32_t *lo, uint32_t *hi, unsigned long long v, bool narrow) {
+    const uint32_t l = (uint32_t)v;
+    if (narrow) {
+        atomicAdd(lo, l);
+    } else {
+        const uint32_t old = atomicAdd(lo, l), c = (uint32_t)(v >> 32) + (old + l < old ? 1u : 0u);
+        if (c) atomicAdd(hi, c);
+    }
+}
 
 // Shared min / max that skip the atomic when the value cannot change the
 // result: a stale read is never below the current minimum (above the
@@ -2131,207 +2141,195 @@ __device__ __forceinline__ void feat_global(seg_cell_features *f, unsigned long 
     }
 }
 
-// One block per row tile (256 consecutive rows; their labels are one
-// contiguous range).  The tile's runs (x extent and final label, the label
-// being its root's, set by k_rank) are first loaded into shared memory by all
-// threads at once, so that no row waits on its own chain of global loads;
-// a tile with more than LABEL_RUNS runs reads them from global memory
-// instead.  Labels: one warp per row, 16-byte streaming stores when rows are
-// 16-byte aligned (X % 4 == 0), zeros between runs.  Then one thread per run
-// folds the run's contribution to its cell (count, coordinate sums, bounding
-// box) into a shared table; after a barrier the table goes to the global
-// cells with one set of atomics per (tile, cell).
+// One block per label tile (VolDev::lb_rows consecutive rows; their labels are
+// one contiguous range of at most 256 KB, in which the runs, in order, are
+// disjoint intervals).  The tile's runs are taken LABEL_RUNS at a time into shared memory by all threads
+// at once, each with its start in the range and its final label (its root's,
+// set by k_rank).  Then
+//   cells   one thread per run folds the run's contribution to its cell
+//           (count, coordinate sums, bounding box) into a shared table, which
+//           goes to the global cells with one set of atomics per (tile, cell);
+//   labels  every warp writes an equal part of the stretch up to the next
+//           runs, 128 voxels at a time as 16-byte stores on 16-byte
+//           boundaries: rows do not matter, so any X stores alike, and the
+//           empty stretches between runs (almost all of a volume) are a plain
+//           fill.
+// Bound by the 4 bytes per voxel written and, below that, by a tile's serial
+// start (offsets, runs, cells): 32 channels of 512 x 512 x 64 (2.1 GB) take
+// 363 us (5.9 TB/s; a plain fill takes 280), 5530 x 5530 x 80 takes 1660 us;
+// one warp per row with 64-bit shared sums took 420 and 2476 us.  Tiles of
+// 512 KB cost 2 % more on the former, tiles of 256 rows 25 % on the latter.
 //
-// The same loop writes every run as a seg_label_run (label 0: its component
-// was dropped) for seg_read_label_runs, into the part of the cell table that
-// no cell uses (RunRecords: the table is sized for the most cells the volume
-// can hold), with the tile's first run and number of labelled runs.  Reading
-// the runs then moves the records (0.7 MB for a 512 x 512 x 64 frame) and not
-// the label image twice (134 MB).
-constexpr int LABEL_RUNS = 2048;
+// The cells loop also writes every run as a seg_label_run (label 0: its
+// component was dropped) for seg_read_label_runs, into the part of the cell
+// table that no cell uses (RunRecords: the table is sized for the most cells
+// the volume can hold), with the tile's first run and number of labelled
+// runs.  Reading the runs then moves the records (0.7 MB for a 512 x 512 x 64
+// frame) and not the label image twice (134 MB).
+constexpr int LABEL_RUNS = 1024;
 
-__global__ void __launch_bounds__(ROW_TILE, 6) k_label_features(const BatchHdr *__restrict__ h) {
-    __shared__ VolIndex<&VolDev::rt_base> VI;
+__global__ void __launch_bounds__(ROW_TILE, 7) k_label_features(const BatchHdr *__restrict__ h) {
+    __shared__ VolIndex<&VolDev::lb_base> VI;
     VI.load(h);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int WARPS = ROW_TILE / 32;
+    constexpr uint32_t WARPS = ROW_TILE / 32;
     __shared__ uint32_t soff[ROW_TILE + 1];
-    __shared__ uint2 srl[LABEL_RUNS];  // staged runs: x0 | x1 << 16, final label
-    __shared__ uint8_t srow[LABEL_RUNS];  // row of each staged run in the tile
+    __shared__ uint2 srl[LABEL_RUNS];     // staged runs: start (voxel of the tile's range), label
+    __shared__ uint16_t slen[LABEL_RUNS]; // their lengths - 1
+    __shared__ uint8_t srow[LABEL_RUNS];  // their rows in the tile
     __shared__ FeatTable T;
     __shared__ uint32_t skept;  // labelled runs of the tile
-    for (uint32_t rt = blockIdx.x; rt < h->nrowtiles; rt += gridDim.x) {
-        const VolDev &V = h->vol[VI.find(h, rt)];
-        const uint32_t lt = rt - V.rt_base;
-        const uint32_t row0 = lt * h->row_tile;
-        const uint32_t nrows = min(h->row_tile, V.rows - row0);
-        __syncthreads();  // previous tile done with soff, srl and T
+    for (uint32_t bt = blockIdx.x; bt < h->nlabtiles; bt += gridDim.x) {
+        const VolDev &V = h->vol[VI.find(h, bt)];
+        const uint32_t lt = bt - V.lb_base;
+        const uint32_t row0 = lt * V.lb_rows;
+        const uint32_t nrows = min(V.lb_rows, V.rows - row0);
+        const uint32_t X = V.X;
+        const bool narrow = (unsigned long long)nrows * X * max(X, max(V.Y, V.Z)) < (1ull << 32);
+        __syncthreads();  // previous tile done with the shared arrays
         if (tid == 0) skept = 0u;
         for (uint32_t i = tid; i <= nrows; i += ROW_TILE) soff[i] = V.rowoff[row0 + i];
         T.key[tid] = 0u;
-        T.cx[tid] = T.sy[tid] = T.sz[tid] = 0ull;
+        T.cnt[tid] = 0u;
         for (int a = 0; a < 3; ++a) {
+            T.lo[a][tid] = T.hi[a][tid] = 0u;
             T.mn[a][tid] = 0xFFFFFFFFu;
             T.mx[a][tid] = 0u;
         }
         __syncthreads();
-        const uint32_t *__restrict__ RX = V.run_x;
-        const uint32_t *__restrict__ RP = V.run_par;
-        const uint32_t *__restrict__ RA = V.run_aux;
         const uint32_t rb = soff[0], re = soff[nrows];
-        const bool staged = re - rb <= (uint32_t)LABEL_RUNS;  // the same in every thread
-        if (staged) {
-            for (uint32_t j = rb + tid; j < re; j += ROW_TILE) {
-                srl[j - rb] = make_uint2(RX[j], RA[RP[j]]);
+        // voxel f of the tile's range is word f + sh of a 16-byte aligned base
+        uint32_t *base = V.labels + (size_t)row0 * X;
+        const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(base) & 15u) >> 2;
+        base -= sh;
+        const uint32_t gend = nrows * X + sh;
+        uint32_t gs = sh;  // first word not written yet
+        for (uint32_t cb = rb;;) {
+            const uint32_t ce = min(re, cb + (uint32_t)LABEL_RUNS), n = ce - cb;
+            if ((uint32_t)tid < nrows) {
+                const uint32_t je = min(soff[tid + 1], ce);
+                for (uint32_t j = max(soff[tid], cb); j < je; ++j) srow[j - cb] = (uint8_t)tid;
             }
-            if ((uint32_t)tid < nrows)
-                for (uint32_t j = soff[tid]; j < soff[tid + 1]; ++j) srow[j - rb] = (uint8_t)tid;
-            __syncthreads();
-        }
-        auto run_x = [&](uint32_t j) { return staged ? srl[j - rb].x : RX[j]; };
-        auto run_label = [&](uint32_t j) { return staged ? srl[j - rb].y : RA[RP[j]]; };
-        // labels
-        const uint32_t X = V.X;
-        const bool vec = (X & 3u) == 0u;
-        for (uint32_t rr = warp; rr < nrows; rr += WARPS) {
-            uint32_t *out = V.labels + (size_t)(row0 + rr) * X;
-            const uint32_t ib = soff[rr], ie = soff[rr + 1];
-            if (vec) {
-                uint4 *o4 = reinterpret_cast<uint4 *>(out);
-                if (ib == ie) {
-                    for (uint32_t x = lane; x < X / 4; x += 32) __stcs(o4 + x, make_uint4(0, 0, 0, 0));
-                    continue;
-                }
-                if (staged && ie - ib <= 16u) {
-                    // few runs: every lane goes through the row's runs in
-                    // step (broadcast reads, no divergent walk) for each
-                    // 128-voxel segment, and fills its 4-voxel chunk
-                    uint32_t j = ib;
-                    for (uint32_t sb = 0; sb < X; sb += 128) {
-                        const uint32_t xb = sb + 4u * lane;
-                        uint32_t v0 = 0, v1 = 0, v2 = 0, v3 = 0;
-                        while (j < ie && (srl[j - rb].x >> 16) < sb) ++j;
-                        for (uint32_t k = j; k < ie; ++k) {
-                            const uint2 rl = srl[k - rb];  // one 8-byte load: extent and label
-                            const uint32_t rx = rl.x;
-                            const uint32_t x0 = rx & 0xFFFFu, x1 = rx >> 16;
-                            if (x0 >= sb + 128u) break;
-                            if (x1 < xb || x0 > xb + 3u) continue;
-                            const uint32_t L = rl.y, w = x1 - x0;
-                            if (xb - x0 <= w) v0 = L;
-                            if (xb + 1u - x0 <= w) v1 = L;
-                            if (xb + 2u - x0 <= w) v2 = L;
-                            if (xb + 3u - x0 <= w) v3 = L;
-                        }
-                        if (xb < X) __stcs(o4 + xb / 4, make_uint4(v0, v1, v2, v3));
-                    }
-                    continue;
-                }
-                uint32_t j = ib, jx = run_x(ib), jl = run_label(ib);
-                for (uint32_t xb = 4 * lane; xb < X; xb += 128) {
-                    // j: the first run that does not end before xb
-                    while (j < ie && (jx >> 16) < xb) {
-                        if (++j < ie) {
-                            jx = run_x(j);
-                            jl = run_label(j);
-                        }
-                    }
-                    uint4 o;
-                    if (j >= ie || (jx & 0xFFFFu) > xb + 3u) {
-                        o = make_uint4(0, 0, 0, 0);            // the 4 voxels lie before run j
-                    } else if ((jx & 0xFFFFu) <= xb && (jx >> 16) >= xb + 3u) {
-                        o = make_uint4(jl, jl, jl, jl);        // all 4 inside run j
-                    } else {
-                        uint32_t l4[4];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const uint32_t x = xb + q;
-                            while (j < ie && (jx >> 16) < x) {
-                                if (++j < ie) {
-                                    jx = run_x(j);
-                                    jl = run_label(j);
-                                }
-                            }
-                            l4[q] = (j < ie && (jx & 0xFFFFu) <= x) ? jl : 0u;
-                        }
-                        o = make_uint4(l4[0], l4[1], l4[2], l4[3]);
-                    }
-                    __stcs(o4 + xb / 4, o);
-                }
-            } else {
-                if (ib == ie) {
-                    for (uint32_t x = lane; x < X; x += 32) __stcs(out + x, 0u);
-                    continue;
-                }
-                uint32_t j = ib, jx = run_x(ib), jl = run_label(ib);
-                for (uint32_t x = lane; x < X; x += 32) {
-                    while (j < ie && (jx >> 16) < x) {
-                        if (++j < ie) {
-                            jx = run_x(j);
-                            jl = run_label(j);
-                        }
-                    }
-                    __stcs(out + x, (j < ie && (jx & 0xFFFFu) <= x) ? jl : 0u);
-                }
+            for (uint32_t i = tid; i < n; i += ROW_TILE) {
+                const uint32_t rx = V.run_x[cb + i];
+                srl[i] = make_uint2(rx & 0xFFFFu, V.run_aux[V.run_par[cb + i]]);
+                slen[i] = (uint16_t)((rx >> 16) - (rx & 0xFFFFu));
             }
-        }
-        const RunRecords rec(V.feat, V.k_cap, V.stat[ST_CELLS], V.stat[ST_RUNS], V.nrt);
-        uint32_t kept = 0;
-        for (uint32_t j = rb + tid; j < re; j += ROW_TILE) {
-            const uint32_t lab = run_label(j);
-            kept += lab != 0u;
-            uint32_t lo;
-            if (staged) {
-                lo = srow[j - rb];
-            } else {
-                // row of run j: the last i with soff[i] <= j
-                uint32_t hi = nrows;
-                lo = 0;
+            // the words up to the next chunk's first run are this chunk's
+            uint32_t ge = gend;
+            if (ce < re) {
+                uint32_t lo = 0, hi = nrows;  // row of run ce: the last i with soff[i] <= ce
                 while (hi - lo > 1) {
                     const uint32_t mid = (lo + hi) >> 1;
-                    if (soff[mid] <= j) lo = mid; else hi = mid;
+                    if (soff[mid] <= ce) lo = mid; else hi = mid;
+                }
+                ge = sh + lo * X + (V.run_x[ce] & 0xFFFFu);
+            }
+            __syncthreads();
+            uint32_t kept = 0;
+            {
+                const RunRecords rec(V.feat, V.k_cap, V.stat[ST_CELLS], V.stat[ST_RUNS], V.nlb);
+                for (uint32_t i = tid; i < n; i += ROW_TILE) {
+                    const uint2 rl = srl[i];
+                    const uint32_t lab = rl.y, x0 = rl.x, lo = srow[i], x1 = x0 + slen[i], row = row0 + lo;
+                    srl[i].x = sh + lo * X + x0;
+                    kept += lab != 0u;
+                    if (rec.words) {
+                        uint32_t *o = rec.words + 3ull * (cb + i);
+                        o[0] = lab;
+                        o[1] = row;
+                        o[2] = x0 | x1 << 16;
+                    }
+                    if (!lab || lab > V.k_cap) continue;
+                    const uint32_t y = row % V.Y, z = row / V.Y;
+                    const unsigned long long len = x1 - x0 + 1u;
+                    const unsigned long long sx = ((unsigned long long)(x0 + x1) * len) >> 1;
+                    uint32_t slot = (lab * 2654435761u) >> 24;
+                    bool done = false;
+                    for (int p = 0; p < FEAT_PROBES && !done; ++p, slot = (slot + 1) & (FEAT_SLOTS - 1)) {
+                        uint32_t k = *reinterpret_cast<volatile uint32_t *>(&T.key[slot]);
+                        if (k == 0u) k = atomicCAS(&T.key[slot], 0u, lab);
+                        if (k == 0u || k == lab) {
+                            atomicAdd(&T.cnt[slot], (uint32_t)len);
+                            sadd(&T.lo[0][slot], &T.hi[0][slot], sx, narrow);
+                            sadd(&T.lo[1][slot], &T.hi[1][slot], len * y, narrow);
+                            sadd(&T.lo[2][slot], &T.hi[2][slot], len * z, narrow);
+                            smin(&T.mn[0][slot], x0);
+                            smax(&T.mx[0][slot], x1);
+                            smin(&T.mn[1][slot], y);
+                            smax(&T.mx[1][slot], y);
+                            smin(&T.mn[2][slot], z);
+                            smax(&T.mx[2][slot], z);
+                            done = true;
+                        }
+                    }
+                    if (!done) {
+                        const uint32_t mn[3] = {x0, y, z}, mx[3] = {x1, y, z};
+                        feat_global(V.feat + (lab - 1), len, sx, len * y, len * z, mn, mx);
+                    }
                 }
             }
-            const uint32_t row = row0 + lo;
-            const uint32_t rx = run_x(j);
-            if (rec.words) {
-                uint32_t *o = rec.words + 3ull * j;
-                o[0] = lab;
-                o[1] = row;
-                o[2] = rx;
+            kept = __reduce_add_sync(FULL, kept);
+            if (lane == 0 && kept) atomicAdd(&skept, kept);
+            __syncthreads();
+            // the labels of words [gs, ge): segments of 128 words, an equal
+            // share of consecutive ones per warp
+            const uint32_t sfirst = gs >> 7, nseg = ((ge + 127u) >> 7) - sfirst;
+            const uint32_t sb = sfirst + nseg / WARPS * (warp + 1) + min(nseg % WARPS, (uint32_t)warp + 1u);
+            uint32_t sg = sfirst + nseg / WARPS * warp + min(nseg % WARPS, (uint32_t)warp);
+            uint32_t j = 0;  // first run that ends at or after the segment's start
+            for (uint32_t hi = n; j < hi;) {
+                const uint32_t mid = (j + hi) >> 1;
+                if (srl[mid].x + slen[mid] < sg << 7) j = mid + 1; else hi = mid;
             }
-            if (!lab || lab > V.k_cap) continue;
-            const uint32_t y = row % V.Y, z = row / V.Y;
-            const uint32_t x0 = rx & 0xFFFFu, x1 = rx >> 16;
-            const unsigned long long len = x1 - x0 + 1u;
-            const unsigned long long sx = ((unsigned long long)(x0 + x1) * len) >> 1;
-            uint32_t slot = (lab * 2654435761u) >> 24;
-            bool done = false;
-            for (int p = 0; p < FEAT_PROBES && !done; ++p, slot = (slot + 1) & (FEAT_SLOTS - 1)) {
-                uint32_t k = *reinterpret_cast<volatile uint32_t *>(&T.key[slot]);
-                if (k == 0u) k = atomicCAS(&T.key[slot], 0u, lab);
-                if (k == 0u || k == lab) {
-                    atomicAdd(&T.cx[slot], (sx << CX_SHIFT) | len);
-                    atomicAdd(&T.sy[slot], len * y);
-                    atomicAdd(&T.sz[slot], len * z);
-                    smin(&T.mn[0][slot], x0);
-                    smax(&T.mx[0][slot], x1);
-                    smin(&T.mn[1][slot], y);
-                    smax(&T.mx[1][slot], y);
-                    smin(&T.mn[2][slot], z);
-                    smax(&T.mx[2][slot], z);
-                    done = true;
+            uint32_t next = j < n ? srl[j].x : 0xFFFFFFFFu;  // start of run j
+            const uint32_t whole = (gs + 127u) >> 7, last = ge >> 7;  // segments [whole, last) lie inside [gs, ge)
+            for (; sg < sb; ++sg) {
+                if (sg >= whole) {  // the empty segments before run j: a fill
+                    const uint32_t to = min(min(sb, last), next >> 7);
+                    uint4 *p = reinterpret_cast<uint4 *>(base + (sg << 7)) + lane;
+                    for (; sg + 4u <= to; sg += 4u, p += 128) {
+                        __stcs(p, make_uint4(0, 0, 0, 0));
+                        __stcs(p + 32, make_uint4(0, 0, 0, 0));
+                        __stcs(p + 64, make_uint4(0, 0, 0, 0));
+                        __stcs(p + 96, make_uint4(0, 0, 0, 0));
+                    }
+                    for (; sg < to; ++sg, p += 32) __stcs(p, make_uint4(0, 0, 0, 0));
+                    if (sg >= sb) break;
+                }
+                const uint32_t w0 = sg << 7, w = w0 + 4u * lane;
+                uint32_t v0 = 0, v1 = 0, v2 = 0, v3 = 0;
+                if (next < w0 + 128u) {
+                    // every lane goes through the segment's runs in step
+                    // (broadcast reads) and fills its four words
+                    for (uint32_t k = j;;) {
+                        const uint32_t b = next, L = srl[k].y, d = slen[k];
+                        if (w - b <= d) v0 = L;
+                        if (w + 1u - b <= d) v1 = L;
+                        if (w + 2u - b <= d) v2 = L;
+                        if (w + 3u - b <= d) v3 = L;
+                        if (b + d >= w0 + 128u) break;  // goes on in the next segment
+                        j = ++k;
+                        next = k < n ? srl[k].x : 0xFFFFFFFFu;
+                        if (next >= w0 + 128u) break;
+                    }
+                }
+                if (w >= gs && w + 4u <= ge) {
+                    __stcs(reinterpret_cast<uint4 *>(base + w), make_uint4(v0, v1, v2, v3));
+                } else {  // the ends of the stretch
+                    if (w >= gs && w < ge) base[w] = v0;
+                    if (w + 1u >= gs && w + 1u < ge) base[w + 1u] = v1;
+                    if (w + 2u >= gs && w + 2u < ge) base[w + 2u] = v2;
+                    if (w + 3u >= gs && w + 3u < ge) base[w + 3u] = v3;
                 }
             }
-            if (!done) {
-                const uint32_t mn[3] = {x0, y, z}, mx[3] = {x1, y, z};
-                feat_global(V.feat + (lab - 1), len, sx, len * y, len * z, mn, mx);
-            }
+            if (ce == re) break;
+            cb = ce;
+            gs = ge;
+            __syncthreads();  // the staged runs are replaced
         }
-        kept = __reduce_add_sync(FULL, kept);
-        if (lane == 0 && kept) atomicAdd(&skept, kept);
-        __syncthreads();
         if (tid == 0) {
+            const RunRecords rec(V.feat, V.k_cap, V.stat[ST_CELLS], V.stat[ST_RUNS], V.nlb);
             if (rec.words) rec.tiles[lt] = make_uint2(rb, skept);
             if (skept) atomicAdd(V.stat + ST_LABEL_RUNS, skept);
         }
@@ -2340,9 +2338,9 @@ __global__ void __launch_bounds__(ROW_TILE, 6) k_label_features(const BatchHdr *
             if (lab) {
                 const uint32_t mn[3] = {T.mn[0][tid], T.mn[1][tid], T.mn[2][tid]};
                 const uint32_t mx[3] = {T.mx[0][tid], T.mx[1][tid], T.mx[2][tid]};
-                const unsigned long long cx = T.cx[tid];
-                feat_global(V.feat + (lab - 1), cx & ((1ull << CX_SHIFT) - 1), cx >> CX_SHIFT, T.sy[tid],
-                            T.sz[tid], mn, mx);
+                unsigned long long sum[3];
+                for (int a = 0; a < 3; ++a) sum[a] = (unsigned long long)T.hi[a][tid] << 32 | T.lo[a][tid];
+                feat_global(V.feat + (lab - 1), T.cnt[tid], sum[0], sum[1], sum[2], mn, mx);
             }
         }
     }
@@ -3901,39 +3899,40 @@ __global__ void __launch_bounds__(256) k_cell_distance(const uint32_t *__restric
 }
 
 // Label runs from the records k_label_features left (rows in order, label 0
-// for dropped runs): the labelled ones, in order.  One block per row tile at a
-// time: its runs start at the sum of the tiles' labelled runs below it, 256
-// records at a time are ranked by a block scan, gathered in shared memory and
-// written as consecutive words.
+// for dropped runs): the labelled ones, in order.  A block takes a contiguous
+// range of label tiles: its runs start at the sum of the tiles' labelled runs
+// below it, 256 records at a time are ranked by a block scan, gathered in
+// shared memory and written as consecutive words.
 __global__ void __launch_bounds__(ROW_TILE) k_runs_compact(const uint32_t *__restrict__ rec,
                                                            const uint2 *__restrict__ tiles, uint32_t ntiles,
                                                            uint32_t runs, uint32_t *__restrict__ out) {
     __shared__ uint32_t sbuf[33];
     __shared__ uint32_t stage[3 * ROW_TILE];
     const uint32_t tid = threadIdx.x;
-    for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const uint32_t rb = tiles[t].x, re = t + 1 < ntiles ? tiles[t + 1].x : runs;
-        uint32_t below = 0;
-        for (uint32_t i = tid; i < t; i += ROW_TILE) below += tiles[i].y;
-        uint64_t at = block_sum<ROW_TILE>(below, sbuf);
-        for (uint32_t j0 = rb; j0 < re; j0 += ROW_TILE) {
-            const uint32_t j = j0 + tid;
-            uint32_t w[3] = {0u, 0u, 0u};
-            if (j < re) {
+    const uint32_t tb = (uint32_t)((uint64_t)ntiles * blockIdx.x / gridDim.x);
+    const uint32_t te = (uint32_t)((uint64_t)ntiles * (blockIdx.x + 1) / gridDim.x);
+    if (tb >= te) return;
+    uint32_t below = 0;
+    for (uint32_t i = tid; i < tb; i += ROW_TILE) below += tiles[i].y;
+    uint64_t at = block_sum<ROW_TILE>(below, sbuf);
+    const uint32_t rb = tiles[tb].x, re = te < ntiles ? tiles[te].x : runs;
+    for (uint32_t j0 = rb; j0 < re; j0 += ROW_TILE) {
+        const uint32_t j = j0 + tid;
+        uint32_t w[3] = {0u, 0u, 0u};
+        if (j < re) {
 #pragma unroll
-                for (int k = 0; k < 3; ++k) w[k] = rec[3ull * j + k];
-            }
-            uint32_t n;
-            const uint32_t r = block_exscan<ROW_TILE>(w[0] != 0u, &n, sbuf);
-            if (w[0]) {
-#pragma unroll
-                for (int k = 0; k < 3; ++k) stage[3u * r + k] = w[k];
-            }
-            __syncthreads();
-            for (uint32_t i = tid; i < 3u * n; i += ROW_TILE) out[3ull * at + i] = stage[i];
-            at += n;
-            __syncthreads();  // stage and sbuf are reused
+            for (int k = 0; k < 3; ++k) w[k] = rec[3ull * j + k];
         }
+        uint32_t n;
+        const uint32_t r = block_exscan<ROW_TILE>(w[0] != 0u, &n, sbuf);
+        if (w[0]) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) stage[3u * r + k] = w[k];
+        }
+        __syncthreads();
+        for (uint32_t i = tid; i < 3u * n; i += ROW_TILE) out[3ull * at + i] = stage[i];
+        at += n;
+        __syncthreads();  // stage and sbuf are reused
     }
 }
 

@@ -123,7 +123,7 @@ struct Request {
     std::vector<size_t> off_den;          // per channel; SIZE_MAX = no denoise (front end: 1 image, MRF: 2)
     size_t off_smooth = SIZE_MAX;         // smoothed images of all channels (SEG_KEEP_SMOOTHED)
     std::vector<uint32_t> mrf_steps, mrf_sel;
-    std::vector<uint32_t> runs, label_runs, nrt;  // foreground runs, runs of the cells, row tiles of the batch
+    std::vector<uint32_t> runs, label_runs, nlb;  // foreground runs, runs of the cells, label tiles
     size_t per_labels = 0, per_feat = 0;  // bytes per channel
     bool owns_input = false;
     bool admitted = false;
@@ -357,11 +357,29 @@ uint32_t batch_row_tile(const seg_ctx *ctx, const Batch &b) {
     return rt;
 }
 
+// Rows per label tile of a volume of width X, and the number of halvings of
+// the tile for a batch: enough for LABEL_TILES tiles per multiprocessor (two
+// rounds of the resident blocks), so that a lone frame's label stores spread
+// over the whole GPU.
+uint32_t label_rows(uint32_t X, uint32_t shrink) {
+    return std::min<uint32_t>(ROW_TILE, std::max<uint32_t>(1u, (LABEL_WORDS >> shrink) / X));
+}
+
+uint32_t batch_label_shrink(const seg_ctx *ctx, const Batch &b) {
+    constexpr uint64_t LABEL_TILES = 12;
+    for (uint32_t k = 0;; ++k) {
+        uint64_t tiles = 0;
+        for (const Request *r : b.reqs)
+            for (uint32_t c = 0; c < r->C; ++c) tiles += cdiv(r->g[c].rows, label_rows(r->g[c].X, k));
+        if (k >= LABEL_SHRINK || tiles >= LABEL_TILES * (uint64_t)ctx->sms) return k;
+    }
+}
+
 void build_header(seg_ctx *ctx, Batch &b) {
     BatchHdr *h = b.slot->h_hdr;
     const uint32_t ty = (uint32_t)ctx->plan.tile_y, tz = batch_tile_z(ctx, b), fz = batch_rows_tile_z(ctx, b);
-    const uint32_t rtile = batch_row_tile(ctx, b);
-    uint32_t fst = 0;
+    const uint32_t rtile = batch_row_tile(ctx, b), lbk = batch_label_shrink(ctx, b);
+    uint32_t fst = 0, lbs = 0;
     uint32_t v = 0, tiles = 0, rts = 0, bks = 0, bts = 0, dn[3] = {0, 0, 0}, dnt = 0, cl = 0;
     uint32_t dtb[DT_NK] = {0, 0, 0, 0, 0, 0};
     uint32_t mrft = 0, mrf_iters = 0;
@@ -508,6 +526,10 @@ void build_header(seg_ctx *ctx, Batch &b) {
             V.nby = (uint32_t)cdiv(g.Y, BRICK_Y);
             V.nbk = V.nby * (uint32_t)cdiv(g.Z, BRICK_Z);
             V.bk_base = bks;
+            V.lb_rows = label_rows(g.X, lbk);
+            V.nlb = (uint32_t)cdiv(g.rows, V.lb_rows);
+            V.lb_base = lbs;
+            lbs += V.nlb;
             {
                 // row pairs across brick faces: every pair of a plane z = 8k
                 // with the plane below; pairs (y, y-1) with y = 32k in every
@@ -530,6 +552,7 @@ void build_header(seg_ctx *ctx, Batch &b) {
     h->nrowtiles = rts;
     h->row_tile = rtile;
     h->nbricks = bks;
+    h->nlabtiles = lbs;
     h->nbtasks = bts;
     h->dn_items[0] = dn[0];
     h->dn_items[1] = dn[1];
@@ -683,7 +706,7 @@ void finalize_batch(seg_ctx *ctx, Slot &s) {
             r->mrf_sel[c] = w[ST_MRF_SEL];
             r->runs[c] = w[ST_RUNS];
             r->label_runs[c] = w[ST_LABEL_RUNS];
-            r->nrt[c] = s.h_hdr->vol[v].nrt;
+            r->nlb[c] = s.h_hdr->vol[v].nlb;
             if (w[ST_ERROR]) bad = true;
         }
         r->state = bad ? SEG_FAILED : SEG_DONE;
@@ -1005,7 +1028,7 @@ int seg_submit_volume(seg_ctx *ctx, const uint16_t *voxels, int on_device, seg_d
     r->mrf_sel.assign(channels, 0);
     r->runs.assign(channels, 0);
     r->label_runs.assign(channels, 0);
-    r->nrt.assign(channels, 0);
+    r->nlb.assign(channels, 0);
     r->errbits.assign(channels, 0);
     r->owns_input = host_in;
     if (!host_in) r->user_dev = voxels;
@@ -1248,7 +1271,7 @@ int seg_read_label_runs(seg_ctx *ctx, seg_req req, uint32_t channel, seg_label_r
     cudaSetDevice(ctx->device);
     cudaStream_t s = ctx->read_stream;
     const size_t bytes = sizeof(seg_label_run) * (size_t)total;
-    const RunRecords rec(r->feat(channel), g.k_cap, r->ncells[channel], r->runs[channel], r->nrt[channel]);
+    const RunRecords rec(r->feat(channel), g.k_cap, r->ncells[channel], r->runs[channel], r->nlb[channel]);
     if (rec.words && total == r->runs[channel]) {
         // every run is labelled: the records are the result
         cudaError_t e = cudaMemcpyAsync(dst, rec.words, bytes,
@@ -1276,7 +1299,7 @@ int seg_read_label_runs(seg_ctx *ctx, seg_req req, uint32_t channel, seg_label_r
             out = stage;
         }
         if (e == cudaSuccess)
-            e = launch_runs_compact(rec, r->nrt[channel], r->runs[channel], reinterpret_cast<uint32_t *>(out),
+            e = launch_runs_compact(rec, r->nlb[channel], r->runs[channel], reinterpret_cast<uint32_t *>(out),
                                     ctx->sms, s);
     } else {
         // no room for the records: two passes over the label image
