@@ -46,11 +46,11 @@ constexpr int ROW_TILE_MIN = 32;  // smallest row tile (batches with few rows)
 constexpr uint32_t LABEL_WORDS = 65536;
 constexpr uint32_t LABEL_SHRINK = 4;
 constexpr int HIST_BINS = 65536;
-// Union-find bricks: BRICK_Y x BRICK_Z rows (one thread each) whose runs are
-// united in shared memory when there are at most BRICK_CAP of them.
-constexpr int BRICK_Y = 32;
-constexpr int BRICK_Z = 8;
-constexpr int BRICK_CAP = 2048;
+// Union-find bricks: bk_y x bk_z rows (at most BRICK_ROWS, the block size),
+// whose runs are united in shared memory when there are at most BRICK_CAP of
+// them.
+constexpr int BRICK_ROWS = 256;
+constexpr int BRICK_CAP = 3072;
 
 // One volume-channel inside a batch.  All pointers are device addresses.
 struct VolDev {
@@ -92,11 +92,13 @@ struct VolDev {
     uint32_t lb_rows;         // rows per label tile (at most ROW_TILE)
     uint32_t nlb;             // label tiles
     uint32_t lb_base;         // first flat label-tile index
+    uint32_t bk_y, bk_z;      // rows of a union-find brick along y and z (powers of two)
     uint32_t nby;             // union-find bricks along y
     uint32_t nbk;             // union-find bricks
     uint32_t bk_base;         // first flat brick index
     uint32_t nbt;             // row pairs that cross a brick face (k_union tasks)
-    uint32_t bt_base;         // first flat k_union task index
+    uint32_t bt_base;         // first flat k_union thread index
+    uint32_t bt_lanes;        // log2 of the threads per row pair
     // denoise front end (dn_r > 0); raw then points at dn_out
     const uint16_t *dn_src;   // observed image [Z][Y][X]
     uint16_t *dn_a, *dn_b;    // box-pass ping-pong buffers (the background ends in dn_a)
@@ -161,7 +163,7 @@ struct BatchHdr {
     uint32_t tile_y;     // rows of a smoothing tile
     uint32_t fs_tiles;   // k_smooth_rows tiles over the batch
     uint32_t nbricks;    // union-find bricks over the batch
-    uint32_t nbtasks;    // k_union tasks over the batch
+    uint32_t nbtasks;    // k_union threads over the batch
     uint32_t dn_items[3];// denoise box-pass items per axis over the batch
     uint32_t dn_tiles;   // denoise median tiles over the batch
     uint32_t cl_items;   // closing dilation items over the batch

@@ -1752,19 +1752,17 @@ __global__ void __launch_bounds__(ROW_TILE) k_row_runs(const BatchHdr *__restric
     }
 }
 
-// Sweep two x-sorted run lists and unite every pair at x-distance <= 1
-// (26-adjacency between runs of rows that differ by one in y and/or z).
-__device__ __forceinline__ void unite_rows(uint32_t *P, const uint32_t *__restrict__ RX, uint32_t i,
-                                           uint32_t ie, uint32_t j, uint32_t je, uint32_t *err,
-                                           uint32_t limit) {
-    while (i < ie && j < je) {
-        const uint32_t a = RX[i], b = RX[j];
-        const uint32_t a0 = a & 0xFFFFu, a1 = a >> 16, b0 = b & 0xFFFFu, b1 = b >> 16;
-        if (b1 + 1 < a0) { ++j; continue; }
-        if (a1 + 1 < b0) { ++i; continue; }
-        uf_union(P, i, j, err, limit);
-        if (a1 < b1) ++i; else ++j;
+// Unites run i with the runs of a neighbouring row, [j, je) in order of x, at
+// x-distance <= 1 (26-adjacency between runs of rows that differ by one in y
+// and/or z): the first one that ends at or after x0 - 1 is found by bisection.
+__device__ __forceinline__ void unite_run(uint32_t *P, const uint32_t *__restrict__ RX, uint32_t i, uint32_t j,
+                                          uint32_t je, uint32_t *err, uint32_t limit) {
+    const uint32_t a = RX[i], a0 = a & 0xFFFFu, a1 = a >> 16;
+    for (uint32_t hi = je; j < hi;) {
+        const uint32_t mid = (j + hi) >> 1;
+        if ((RX[mid] >> 16) + 1u < a0) j = mid + 1; else hi = mid;
     }
+    for (; j < je && (RX[j] & 0xFFFFu) <= a1 + 1u; ++j) uf_union(P, i, j, err, limit);
 }
 
 // ---- brick-local union-find in shared memory ------------------------------
@@ -1806,68 +1804,78 @@ __device__ __forceinline__ bool sm_union(volatile uint32_t *P, uint32_t a, uint3
     return false;
 }
 
-__device__ __forceinline__ bool sm_unite_rows(volatile uint32_t *P, const uint32_t *RX, uint32_t i,
-                                              uint32_t ie, uint32_t j, uint32_t je, uint32_t limit) {
+// First of the runs [j, je) of a brick row that ends at or after a0 - 1.
+__device__ __forceinline__ uint32_t sm_first(const uint32_t *RX, uint32_t a0, uint32_t j, uint32_t je) {
+    while (j < je) {
+        const uint32_t mid = (j + je) >> 1;
+        if ((RX[mid] >> 16) + 1u < a0) j = mid + 1; else je = mid;
+    }
+    return j;
+}
+
+// Unites the component of node r (an ancestor of a run of extent a) with those
+// of the runs [j, je) that the run touches, unless r is their parent.
+__device__ __forceinline__ bool sm_unite_run(volatile uint32_t *P, const uint32_t *RX, uint32_t a, uint32_t r,
+                                             uint32_t j, uint32_t je, uint32_t limit) {
     bool ok = true;
-    while (i < ie && j < je) {
-        const uint32_t a = RX[i], b = RX[j];
-        const uint32_t a0 = a & 0xFFFFu, a1 = a >> 16, b0 = b & 0xFFFFu, b1 = b >> 16;
-        if (b1 + 1 < a0) { ++j; continue; }
-        if (a1 + 1 < b0) { ++i; continue; }
-        ok &= sm_union(P, i, j, limit);
-        if (a1 < b1) ++i; else ++j;
+    for (j = sm_first(RX, a & 0xFFFFu, j, je); j < je && (RX[j] & 0xFFFFu) <= (a >> 16) + 1u; ++j) {
+        const uint32_t q = P[j];
+        if (q != r || limit == 0u) ok &= sm_union(P, r, q, limit);
     }
     return ok;
 }
 
-// Every run's parent becomes its root.  Called between barriers, with no
-// union in progress: a concurrent reader sees the old parent or the root,
-// both ancestors of the node.
+// Every run's parent becomes its root, by pointer jumping (a chain of k links
+// takes log2 k rounds).  Called by the whole block between barriers, with no
+// union in progress: a concurrent reader sees the old parent or a higher
+// ancestor.
 __device__ __forceinline__ void sm_compress(volatile uint32_t *P, uint32_t n, uint32_t t, uint32_t nt) {
-    for (uint32_t l = t; l < n; l += nt) {
-        uint32_t r = P[l];
-        if (r == l) continue;
-        uint32_t p = P[r];
-        while (p != r) {
-            r = p;
-            p = P[r];
+    bool more = true;
+    while (__syncthreads_or(more)) {
+        more = false;
+        for (uint32_t l = t; l < n; l += nt) {
+            const uint32_t p = P[l], g = P[p];
+            if (g != p) {
+                P[l] = g;
+                more = true;
+            }
         }
-        P[l] = r;
     }
 }
 
-// Global run index of local run l: the brick's runs of z-plane lz are one
-// contiguous global range starting at gb[lz] (local start soff[lz * BRICK_Y]).
-__device__ __forceinline__ uint32_t brick_global(uint32_t l, const uint32_t *soff, const uint32_t *gb) {
-    uint32_t lz = 0;
-#pragma unroll
-    for (int k = 1; k < BRICK_Z; ++k) lz = soff[k * BRICK_Y] <= l ? (uint32_t)k : lz;
-    return gb[lz] + (l - soff[lz * BRICK_Y]);
-}
-
-// One block per brick of BRICK_Y x BRICK_Z rows, one thread per row.  The
-// brick's runs are copied to shared memory, every 26-adjacent pair of runs
-// whose rows both lie in the brick is united there, and each run's global
-// parent is set to its local root (a valid union-find state: the parent is
-// a lower run of the same component).  A brick with more than BRICK_CAP runs
-// unites the same pairs through the global structure instead; that touches
-// only the brick's own runs, so it cannot interfere with other bricks.
-// k_union then unites the pairs of rows that lie in different bricks.
-__global__ void __launch_bounds__(BRICK_Y * BRICK_Z) k_union_local(const BatchHdr *__restrict__ h) {
+// One block per brick of bk_y x bk_z rows.  The brick's runs are copied to
+// shared memory, every 26-adjacent pair of runs whose rows both lie in the
+// brick is united there, and each run's global parent is set to its local root
+// (a valid union-find state: the parent is a lower run of the same component).
+// One thread per run, not per row, so that rows of many runs do not wait for
+// one thread's walk; bricks of wide volumes have fewer rows, so that their runs
+// fit.  Bound by the latency of shared-memory chains between the barriers: 83 us
+// for 32 channels of 512 x 512 x 64 and 230 us for 5530 x 5530 x 80 (one thread
+// per row of 32 x 8-row bricks: 320 and 2920 us, a few bricks past their capacity
+// and long serial walks).  3072 runs and 128 K voxels a brick: with 2048 runs
+// crowded bricks overflow (270 us), with 4096 fewer blocks are resident (145 us).
+// A
+// brick with more than BRICK_CAP runs unites the same pairs through the global
+// structure instead, run by run too; that touches only the brick's own runs, so
+// it cannot interfere with other bricks.  k_union then unites the pairs of rows that lie
+// in different bricks.
+__global__ void __launch_bounds__(BRICK_ROWS) k_union_local(const BatchHdr *__restrict__ h) {
     __shared__ VolIndex<&VolDev::bk_base> VI;
     VI.load(h);
-    constexpr int NT = BRICK_Y * BRICK_Z;
+    constexpr uint32_t NT = BRICK_ROWS;
     __shared__ uint32_t sx[BRICK_CAP];       // run x0 | x1 << 16
     __shared__ uint32_t sp[BRICK_CAP];       // local parent
-    __shared__ uint32_t soff[NT + 1];        // local run offset of each brick row
-    __shared__ uint32_t gb[BRICK_Z];         // global index of each plane's first run
+    __shared__ uint8_t srow[BRICK_CAP];      // brick row of the run
+    __shared__ uint32_t soff[NT + 2];        // local run offset of each brick row (and past the last one)
+    __shared__ uint32_t gofs[NT];            // global minus local run index of each brick row
     __shared__ uint32_t sbuf[33];
-    const uint32_t t = threadIdx.x, ly = t % BRICK_Y, lz = t / BRICK_Y;
+    const uint32_t t = threadIdx.x;
     for (uint32_t bk = blockIdx.x; bk < h->nbricks; bk += gridDim.x) {
         const VolDev &V = h->vol[VI.find(h, bk)];
-        const uint32_t lb = bk - V.bk_base;
-        const uint32_t y = (lb % V.nby) * BRICK_Y + ly, z = (lb / V.nby) * BRICK_Z + lz;
-        const bool valid = y < V.Y && z < V.Z;
+        const uint32_t lb = bk - V.bk_base, BY = V.bk_y, nr = BY * V.bk_z;
+        const uint32_t ly = t % BY, lz = t / BY;
+        const uint32_t y = (lb % V.nby) * BY + ly, z = (lb / V.nby) * V.bk_z + lz;
+        const bool valid = t < nr && y < V.Y && z < V.Z;
         const uint32_t row = z * V.Y + y;
         uint32_t ib = 0, cnt = 0;
         if (valid) {
@@ -1879,61 +1887,71 @@ __global__ void __launch_bounds__(BRICK_Y * BRICK_Z) k_union_local(const BatchHd
         // the previous iteration's reads
         const uint32_t loc = block_exscan<NT>(cnt, &n, sbuf);
         if (n == 0) continue;  // n is the same in every thread
+        const uint32_t lim = V.union_limit;
+        soff[t] = loc;
+        gofs[t] = ib - loc;
+        if (t == NT - 1) soff[NT] = soff[NT + 1] = n;
         if (n > (uint32_t)BRICK_CAP) {
-            if (cnt) {
-                const uint32_t ie = ib + cnt, lim = V.union_limit;
-                uint32_t *err = V.stat + ST_ERROR;
-                if (ly > 0) unite_rows(V.run_par, V.run_x, ib, ie, V.rowoff[row - 1], ib, err, lim);
-                if (lz > 0) {
-                    const uint32_t rz = row - V.Y;
-                    if (ly > 0)
-                        unite_rows(V.run_par, V.run_x, ib, ie, V.rowoff[rz - 1], V.rowoff[rz], err, lim);
-                    unite_rows(V.run_par, V.run_x, ib, ie, V.rowoff[rz], V.rowoff[rz + 1], err, lim);
-                    if (ly + 1 < (uint32_t)BRICK_Y && y + 1 < V.Y)
-                        unite_rows(V.run_par, V.run_x, ib, ie, V.rowoff[rz + 1], V.rowoff[rz + 2], err, lim);
+            __syncthreads();
+            uint32_t *err = V.stat + ST_ERROR;
+            for (uint32_t l = t; l < n; l += NT) {
+                uint32_t r = 0;  // brick row of run l: the last one with soff <= l
+                for (uint32_t hi = nr; hi - r > 1u;) {
+                    const uint32_t m = (r + hi) >> 1;
+                    if (soff[m] <= l) r = m; else hi = m;
+                }
+                auto unite = [&](uint32_t q) {  // with the runs of brick row q
+                    unite_run(V.run_par, V.run_x, l + gofs[r], soff[q] + gofs[q], soff[q + 1] + gofs[q], err, lim);
+                };
+                const uint32_t ry = r % BY;
+                if (ry) unite(r - 1);
+                if (r >= BY) {
+                    if (ry) unite(r - BY - 1);
+                    unite(r - BY);
+                    if (ry + 1 < BY) unite(r - BY + 1);
                 }
             }
             continue;
         }
-        soff[t] = loc;
-        if (t == NT - 1) soff[NT] = n;
-        if (ly == 0) gb[lz] = ib;
-        // Each warp holds one plane of the brick (32 rows): it stages its own
-        // runs and unites its rows with their (y-1) neighbours, which lie in
-        // the same plane, synchronising with __syncwarp only.
-        const uint32_t pbeg = __shfl_sync(FULL, loc, 0), pend = __shfl_sync(FULL, loc + cnt, 31);
-        const uint32_t pg = __shfl_sync(FULL, ib, 0);  // global index of the plane's first run
-        for (uint32_t l = pbeg + ly; l < pend; l += BRICK_Y) {
-            sx[l] = V.run_x[pg + (l - pbeg)];
+        for (uint32_t l = loc; l < loc + cnt; ++l) srow[l] = (uint8_t)t;
+        __syncthreads();
+        for (uint32_t l = t; l < n; l += NT) {
+            sx[l] = V.run_x[l + gofs[srow[l]]];
             sp[l] = l;
         }
-        __syncwarp();
-        // Three phases, each followed by a full compression (every run points
-        // at its root) so that no phase walks long paths: rows of one plane,
-        // then the same row of the plane below, then the two diagonals.
-        const uint32_t i1 = loc + cnt, lim = V.union_limit, u = t - BRICK_Y;
+        __syncthreads();
+        // Three phases, each followed by a compression (every run points at
+        // its root), so that the next one sees at once which pairs are united
+        // already: rows of one plane ...
         bool ok = true;
-        if (cnt && ly > 0) ok &= sm_unite_rows(sp, sx, loc, i1, soff[t - 1], soff[t], lim);  // (y-1, z)
-        __syncwarp();
-        for (uint32_t l = pbeg + ly; l < pend; l += BRICK_Y) {  // compress this plane's runs
-            uint32_t r = sp[l];
-            if (r == l) continue;
-            uint32_t q = sp[r];
-            while (q != r) {
-                r = q;
-                q = sp[r];
+        for (uint32_t l = t; l < n; l += NT) {
+            const uint32_t r = srow[l];
+            if (r % BY == 0u) continue;
+            const uint32_t a = sx[l], je = soff[r];
+            uint32_t j = sm_first(sx, a & 0xFFFFu, soff[r - 1], je);
+            if (j >= je || (sx[j] & 0xFFFFu) > (a >> 16) + 1u) continue;
+            if (lim) {
+                // the first link needs no root: j is lower than l
+                const uint32_t old = atomicMin(sp + l, j);
+                if (old != l) ok &= sm_union(sp, old, j, lim);
+                ++j;
             }
-            sp[l] = r;
+            for (; j < je && (sx[j] & 0xFFFFu) <= (a >> 16) + 1u; ++j) ok &= sm_union(sp, l, j, lim);
         }
-        __syncthreads();
-        if (cnt && lz > 0) ok &= sm_unite_rows(sp, sx, loc, i1, soff[u], soff[u + 1], lim);  // (y, z-1)
-        __syncthreads();
         sm_compress(sp, n, t, NT);
-        __syncthreads();
-        if (cnt && lz > 0) {
-            if (ly > 0) ok &= sm_unite_rows(sp, sx, loc, i1, soff[u - 1], soff[u], lim);     // (y-1, z-1)
-            if (ly + 1 < (uint32_t)BRICK_Y)
-                ok &= sm_unite_rows(sp, sx, loc, i1, soff[u + 1], soff[u + 2], lim);         // (y+1, z-1)
+        // ... the same row of the plane below ...
+        for (uint32_t l = t; l < n; l += NT) {
+            const uint32_t r = srow[l];
+            if (r >= BY) ok &= sm_unite_run(sp, sx, sx[l], sp[l], soff[r - BY], soff[r - BY + 1], lim);
+        }
+        sm_compress(sp, n, t, NT);
+        // ... and its two diagonals
+        for (uint32_t l = t; l < n; l += NT) {
+            const uint32_t r = srow[l];
+            if (r < BY) continue;
+            const uint32_t u = r - BY, ry = r % BY;
+            if (ry) ok &= sm_unite_run(sp, sx, sx[l], sp[l], soff[u - 1], soff[u], lim);
+            if (ry + 1 < BY) ok &= sm_unite_run(sp, sx, sx[l], sp[l], soff[u + 1], soff[u + 2], lim);
         }
         if (!ok) atomicOr(V.stat + ST_ERROR, ERR_UNION);
         __syncthreads();
@@ -1943,57 +1961,112 @@ __global__ void __launch_bounds__(BRICK_Y * BRICK_Z) k_union_local(const BatchHd
                 r = p;
                 p = sp[r];
             }
-            V.run_par[brick_global(l, soff, gb)] = brick_global(r, soff, gb);
+            V.run_par[l + gofs[srow[l]]] = r + gofs[srow[r]];
         }
     }
 }
 
-// One thread per pair of 26-adjacent rows that lie in different bricks, in
-// four groups (row y, plane z; neighbour rows (y-1,z), (y-1,z-1), (y,z-1),
-// (y+1,z-1)):
-//   planes z = 8k > 0: every row with each of its three neighbours in z-1;
-//   rows y = 32k > 0, every plane: (y-1, z);
-//   rows y = 32k > 0, the other planes z > 0: (y-1, z-1);
-//   rows y = 32k - 1 (y+1 < Y), the other planes z > 0: (y+1, z-1).
-// Consecutive threads take consecutive rows of a plane where they can.
+// 2^bt_lanes threads (more for wide rows) per pair of 26-adjacent rows that lie
+// in different bricks, each with every 2^bt_lanes-th run of the first; four
+// groups (row y, plane z; neighbour rows (y-1,z), (y-1,z-1), (y,z-1),
+// (y+1,z-1); bricks of BY x BZ rows):
+//   planes z = k BZ > 0: every row with each of its three neighbours in z-1;
+//   rows y = k BY > 0, every plane: (y-1, z);
+//   rows y = k BY > 0, the other planes z > 0: (y-1, z-1);
+//   rows y = k BY - 1 (y+1 < Y), the other planes z > 0: (y+1, z-1).
+// Consecutive threads take consecutive rows of a plane where they can.  After
+// k_union_local a run's parent is its brick's root of the component, and the
+// many runs with which a component crosses a face give the same pair of
+// parents: a warp's lanes step through their touching runs together, one lane
+// unites each distinct pair, and pairs united before are remembered per block
+// in a small table (a pair is tagged with 27 bits for either run and 10 for
+// the volume), so that the unions, whose atomics and root walks otherwise
+// collide, are few (42 against 83 us for 32 channels of 512 x 512 x 64).
 __global__ void __launch_bounds__(ROW_TILE) k_union(const BatchHdr *__restrict__ h) {
     __shared__ VolIndex<&VolDev::bt_base> VI;
+    __shared__ unsigned long long pairs[512];
+    for (uint32_t i = threadIdx.x; i < 512u; i += ROW_TILE) pairs[i] = 0ull;
     VI.load(h);
-    const uint32_t stride = gridDim.x * blockDim.x;
-    for (uint32_t gt = blockIdx.x * blockDim.x + threadIdx.x; gt < h->nbtasks; gt += stride) {
-        const VolDev &V = h->vol[VI.find(h, gt)];
-        uint32_t t = gt - V.bt_base;
-        const uint32_t Y = V.Y, Z = V.Z;
-        const uint32_t nzb = (Z - 1) / BRICK_Z, nyb = (Y - 1) / BRICK_Y, nzi = Z - 1 - nzb;
+    const uint32_t stride = gridDim.x * blockDim.x, wl = threadIdx.x & 31u, nt = h->nbtasks;
+    for (uint32_t g0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); g0 < nt; g0 += stride) {
+        const uint32_t gt = min(g0 + wl, nt - 1u), vi = VI.find(h, gt);
+        const VolDev &V = h->vol[vi];
+        const uint32_t step = 1u << V.bt_lanes, lane = (gt - V.bt_base) & (step - 1u);
+        uint32_t t = (gt - V.bt_base) >> V.bt_lanes;
+        const uint32_t Y = V.Y, Z = V.Z, BY = V.bk_y, BZ = V.bk_z;
+        const uint32_t nzb = (Z - 1) / BZ, nyb = (Y - 1) / BY, nzi = Z - 1 - nzb;
         uint32_t y, z, nb;
         if (t < nzb * Y * 3) {
             const uint32_t pz = t / (3 * Y), rem = t - pz * 3 * Y;
-            z = BRICK_Z * (pz + 1);
+            z = BZ * (pz + 1);
             nb = 1 + rem / Y;
             y = rem % Y;
         } else {
             t -= nzb * Y * 3;
             if (t < nyb * Z) {
                 z = t / nyb;
-                y = BRICK_Y * (t % nyb + 1);
+                y = BY * (t % nyb + 1);
                 nb = 0;
             } else {
                 t -= nyb * Z;
-                const uint32_t grp = t / (nyb * nzi);  // 0: (y-1, z-1) at y = 32k; 1: (y+1, z-1) at 32k - 1
+                const uint32_t grp = t / (nyb * nzi);  // 0: (y-1, z-1) at y = k BY; 1: (y+1, z-1) at k BY - 1
                 t -= grp * nyb * nzi;
                 const uint32_t iz = t / nyb;
-                z = iz + 1 + iz / (BRICK_Z - 1);  // the iz-th plane with z % 8 != 0, z > 0
-                y = BRICK_Y * (t % nyb + 1) - grp;
+                z = iz + 1 + iz / (BZ - 1);  // the iz-th plane with z % BZ != 0, z > 0
+                y = BY * (t % nyb + 1) - grp;
                 nb = grp ? 3u : 1u;
             }
         }
-        if (nb == 1 && y == 0) continue;
-        if (nb == 3 && y + 1 >= Y) continue;
-        const uint32_t row = z * Y + y;
-        const uint32_t ib = V.rowoff[row], ie = V.rowoff[row + 1];
-        if (ib == ie) continue;
-        const uint32_t r = nb == 0 ? row - 1 : row - Y + nb - 2;
-        unite_rows(V.run_par, V.run_x, ib, ie, V.rowoff[r], V.rowoff[r + 1], V.stat + ST_ERROR, V.union_limit);
+        const bool pair = g0 + wl < nt && !(nb == 1 && y == 0) && !(nb == 3 && y + 1 >= Y);
+        uint32_t i = 0, ie = 0, j = 0, je = 0;
+        if (pair) {
+            const uint32_t row = z * Y + y, r = nb == 0 ? row - 1 : row - Y + nb - 2;
+            i = V.rowoff[row] + lane;
+            ie = V.rowoff[row + 1];
+            if (i < ie) {
+                j = V.rowoff[r];
+                je = V.rowoff[r + 1];
+                if (j == je) ie = 0;
+            }
+        }
+        if (!__any_sync(FULL, i < ie)) continue;
+        const bool tag = vi < 1024u && V.stat[ST_RUNS] < 1u << 27;
+        uint32_t a = 0, k = 0;
+        auto first = [&]() {  // the first run of [j, je) that ends at or after run i's x0 - 1
+            a = V.run_x[i];
+            k = j;
+            for (uint32_t hi = je; k < hi;) {
+                const uint32_t mid = (k + hi) >> 1;
+                if ((V.run_x[mid] >> 16) + 1u < (a & 0xFFFFu)) k = mid + 1; else hi = mid;
+            }
+        };
+        if (i < ie) first();
+        for (;;) {
+            // this lane's next touching run k
+            while (i < ie && (k >= je || (V.run_x[k] & 0xFFFFu) > (a >> 16) + 1u)) {
+                i += step;
+                if (i < ie) first();
+            }
+            const bool touch = i < ie;
+            if (!__any_sync(FULL, touch)) break;
+            uint32_t p = 0, q = 0;
+            if (touch) {
+                p = __ldcg(V.run_par + i);
+                q = __ldcg(V.run_par + k);
+                ++k;
+            }
+            const unsigned long long key = ((unsigned long long)p << 27 | q) << 10 | vi;  // not 0 when p != q
+            volatile unsigned long long *seen = pairs + ((p * 2654435761u ^ q * 2246822519u) >> 23);
+            const bool need = p != q && !(tag && *seen == key);
+            // the lanes that need this pair united (an untagged lane: itself)
+            uint32_t same = __match_any_sync(FULL, key) & __ballot_sync(FULL, need && tag);
+            if (!tag) same = 1u << wl;
+            if (need && wl == (uint32_t)__ffs(same) - 1u) {
+                uf_union(V.run_par, p, q, V.stat + ST_ERROR, V.union_limit);
+                if (tag) *seen = key;
+            }
+            __syncwarp();
+        }
     }
 }
 
@@ -4110,7 +4183,7 @@ cudaError_t configure_kernels(int device, LaunchPlan &plan) {
     if ((e = resident((const void *)k_keep_count, ROW_TILE, &g2)) != cudaSuccess) return e;
     if ((e = resident((const void *)k_rank, ROW_TILE, &g3)) != cudaSuccess) return e;
     plan.grid_rows = std::min(g1, std::min(g2, g3));
-    if ((e = resident((const void *)k_union_local, BRICK_Y * BRICK_Z, &plan.grid_ul)) != cudaSuccess) return e;
+    if ((e = resident((const void *)k_union_local, BRICK_ROWS, &plan.grid_ul)) != cudaSuccess) return e;
     if ((e = resident((const void *)k_union, ROW_TILE, &g1)) != cudaSuccess) return e;
     if ((e = resident((const void *)k_flatten, ROW_TILE, &g2)) != cudaSuccess) return e;
     plan.grid_task = std::min(g1, g2);
@@ -4272,7 +4345,7 @@ cudaError_t launch_pipeline(const BatchHdr *d, const LaunchPlan &p, cudaStream_t
     rec();
     k_row_runs<<<p.grid_rows, ROW_TILE, 0, s>>>(d);
     rec();
-    k_union_local<<<p.grid_ul, BRICK_Y * BRICK_Z, 0, s>>>(d);
+    k_union_local<<<p.grid_ul, BRICK_ROWS, 0, s>>>(d);
     rec();
     k_union<<<p.grid_task, ROW_TILE, 0, s>>>(d);
     rec();

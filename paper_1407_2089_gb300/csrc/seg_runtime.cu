@@ -357,6 +357,34 @@ uint32_t batch_row_tile(const seg_ctx *ctx, const Batch &b) {
     return rt;
 }
 
+// Rows of a union-find brick: 32 x 8, halved along y and z in turn while the
+// brick spans more than `voxels` voxels, so that its runs (about one per 300
+// voxels on microscope data, up to one per 50 among vessels) fit in shared
+// memory for wide volumes too.
+void brick_shape(uint32_t X, uint64_t voxels, uint32_t &by, uint32_t &bz) {
+    by = 32;
+    bz = 8;
+    while ((uint64_t)by * bz * X > voxels && by > 4) {
+        if (by > 2 * bz) by /= 2; else bz /= 2;
+    }
+}
+
+// Brick size of a batch: 128 K voxels (fewest unions across bricks), halved
+// for batches with fewer than eight bricks (a full set of resident blocks) per
+// multiprocessor, which would wait for their fullest brick.
+uint64_t batch_brick_voxels(const seg_ctx *ctx, const Batch &b) {
+    constexpr uint64_t MOST = 131072, LEAST = 32768;
+    for (uint64_t v = MOST;; v /= 2) {
+        uint64_t bricks = 0;
+        for (const Request *r : b.reqs) {
+            uint32_t by, bz;
+            brick_shape(r->dims.x, v, by, bz);
+            bricks += r->C * cdiv(r->dims.y, by) * cdiv(r->dims.z, bz);
+        }
+        if (v <= LEAST || bricks >= 8ull * (uint64_t)ctx->sms) return v;
+    }
+}
+
 // Rows per label tile of a volume of width X, and the number of halvings of
 // the tile for a batch: enough for LABEL_TILES tiles per multiprocessor (two
 // rounds of the resident blocks), so that a lone frame's label stores spread
@@ -379,6 +407,7 @@ void build_header(seg_ctx *ctx, Batch &b) {
     BatchHdr *h = b.slot->h_hdr;
     const uint32_t ty = (uint32_t)ctx->plan.tile_y, tz = batch_tile_z(ctx, b), fz = batch_rows_tile_z(ctx, b);
     const uint32_t rtile = batch_row_tile(ctx, b), lbk = batch_label_shrink(ctx, b);
+    const uint64_t bkv = batch_brick_voxels(ctx, b);
     uint32_t fst = 0, lbs = 0;
     uint32_t v = 0, tiles = 0, rts = 0, bks = 0, bts = 0, dn[3] = {0, 0, 0}, dnt = 0, cl = 0;
     uint32_t dtb[DT_NK] = {0, 0, 0, 0, 0, 0};
@@ -523,19 +552,20 @@ void build_header(seg_ctx *ctx, Batch &b) {
             V.nrt = (uint32_t)cdiv(g.rows, rtile);
             V.tile_base = tiles;
             V.rt_base = rts;
-            V.nby = (uint32_t)cdiv(g.Y, BRICK_Y);
-            V.nbk = V.nby * (uint32_t)cdiv(g.Z, BRICK_Z);
+            brick_shape(g.X, bkv, V.bk_y, V.bk_z);
+            V.nby = (uint32_t)cdiv(g.Y, V.bk_y);
+            V.nbk = V.nby * (uint32_t)cdiv(g.Z, V.bk_z);
             V.bk_base = bks;
             V.lb_rows = label_rows(g.X, lbk);
             V.nlb = (uint32_t)cdiv(g.rows, V.lb_rows);
             V.lb_base = lbs;
             lbs += V.nlb;
             {
-                // row pairs across brick faces: every pair of a plane z = 8k
-                // with the plane below; pairs (y, y-1) with y = 32k in every
-                // plane; the two diagonals through y = 32k and y = 32k - 1 in
-                // the other planes
-                const uint32_t nzb = (g.Z - 1) / BRICK_Z, nyb = (g.Y - 1) / BRICK_Y;
+                // row pairs across brick faces: every pair of a plane
+                // z = k bk_z with the plane below; pairs (y, y-1) with
+                // y = k bk_y in every plane; the two diagonals through
+                // y = k bk_y and y = k bk_y - 1 in the other planes
+                const uint32_t nzb = (g.Z - 1) / V.bk_z, nyb = (g.Y - 1) / V.bk_y;
                 const uint32_t nzi = g.Z - 1 - nzb;
                 V.nbt = nzb * g.Y * 3 + nyb * g.Z + 2 * nyb * nzi;
             }
@@ -543,7 +573,11 @@ void build_header(seg_ctx *ctx, Batch &b) {
             tiles += V.ntx * V.nty * V.ntz;
             rts += V.nrt;
             bks += V.nbk;
-            bts += V.nbt;
+            // about one thread per run of a row (one run per 400 voxels on
+            // microscope data)
+            V.bt_lanes = 0;
+            while (V.bt_lanes < 5u && (512u << V.bt_lanes) < g.X) ++V.bt_lanes;
+            bts += V.nbt << V.bt_lanes;
         }
     }
     h->nvol = v;
