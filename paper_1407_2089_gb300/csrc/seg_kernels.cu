@@ -1111,10 +1111,14 @@ struct FsSync {
 
 // One tile: octets [x0, x0 + 8 rte) of rows [y0, y0 + TYF) of planes [z0, z1).
 // RTC = FS_RT: rows of 64 octets (8 rows per tile), HXC: halo chunks
-// (x-tiled rows), both known at compile time; RTC = 0: the shape of V.
+// (x-tiled rows), both known at compile time; RTC = 0: the shape of V.  RAG: 0
+// for rows of X % 8 == 0 voxels; else rows start 4-byte aligned only (4-byte
+// copies and stores), and 2 for the tile at the row's end, whose last octet is
+// partial (only it pays for testing every voxel).
 template <int RTC, int HXC, int RAG>
 __device__ __forceinline__ void smooth_rows_tile(const VolDev &V, uint32_t ix, uint32_t iy, int z0, int z1,
                                                  unsigned char *ring, uint32_t *sh, FsSync &S) {
+    constexpr bool PART = RAG == 2;
     const int tid = threadIdx.x, lane = tid & 31;
     const int X = (int)V.X, Y = (int)V.Y, Z = (int)V.Z;
     // the descriptor's fields in registers (the barrier operations below are
@@ -1141,7 +1145,7 @@ __device__ __forceinline__ void smooth_rows_tile(const VolDev &V, uint32_t ix, u
     const bool emit_ok = act && y0 + ty < Y;
     const bool haloL = x0 > 0, haloR = x0 + 8 * rte < X;
     const bool edgeL = q == 0, edgeR = q == rte - 1;
-    const int nvl = RAG && edgeR ? min(8, X - (x0 + 8 * q)) : 8;  // valid voxels of this lane's octet
+    const int nvl = PART && edgeR ? min(8, X - (x0 + 8 * q)) : 8;  // valid voxels of this lane's octet
     // neighbour words this lane y-sums itself: at a warp's ends and at the
     // tile's ends of x-tiled rows (the halo chunks)
     const bool ownL = edgeL ? haloL : lane == 0;
@@ -1257,22 +1261,32 @@ __device__ __forceinline__ void smooth_rows_tile(const VolDev &V, uint32_t ix, u
             }
             const uint32_t nl = __shfl_up_sync(FULL, yw[3], 1);
             const uint32_t nr = __shfl_down_sync(FULL, yw[0], 1);
-            uint32_t v[12];
+            // x pass: p[j] = v[j] + 4 v[j+1] + 6 v[j+2] + 4 v[j+3] + v[j+4] over the
+            // y-sums v[0..11] of the octet and two voxels on either side
+            uint32_t p[8];
             if (!__any_sync(FULL, act && (chk & 0xF000F000u) != 0u)) {
                 const uint32_t wl = ownL ? hw : (edgeL ? __byte_perm(yw[0], 0u, 0x1010u) : nl);
                 const uint32_t wr = ownR ? hw : (edgeR ? __byte_perm(yw[3], 0u, 0x3232u) : nr);
-                v[0] = wl & 0xFFFFu;
-                v[1] = wl >> 16;
-    #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    v[2 + 2 * i] = yw[i] & 0xFFFFu;
-                    v[3 + 2 * i] = yw[i] >> 16;
+                // y-sums as they are packed, two of them and their weights per
+                // 16 x 8-bit dot product
+                uint32_t w[6] = {wl, yw[0], yw[1], yw[2], yw[3], wr};
+                if (PART && nvl < 8) {
+                    // the row's last octet is partial (nvl = 2, 4 or 6 for even
+                    // X): the voxels past the end repeat the last one
+                    const uint32_t e = __byte_perm(nvl <= 2 ? w[1] : (nvl <= 4 ? w[2] : w[3]), 0u, 0x3232u);
+#pragma unroll
+                    for (int k = 2; k < 6; ++k)
+                        if (2 * k >= 2 + nvl) w[k] = e;
                 }
-                v[10] = wr & 0xFFFFu;
-                v[11] = wr >> 16;
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    p[2 * m] = __dp2a_lo(w[m], 0x0401u, __dp2a_lo(w[m + 1], 0x0406u, w[m + 2] & 0xFFFFu));
+                    p[2 * m + 1] = __dp2a_lo(w[m + 2], 0x0104u, __dp2a_lo(w[m + 1], 0x0604u, w[m] >> 16));
+                }
             } else {
                 // a raw value of 4096 or more in this warp's part of the plane:
                 // its y pass again, in 32-bit lanes
+                uint32_t v[12];
     #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const unsigned char *wp = cp + 4 * i;
@@ -1295,32 +1309,31 @@ __device__ __forceinline__ void smooth_rows_tile(const VolDev &V, uint32_t ix, u
                 v[1] = ownL ? hhi : (edgeL ? v[2] : l1);
                 v[10] = ownR ? hlo : (edgeR ? v[9] : q0);
                 v[11] = ownR ? hhi : (edgeR ? v[9] : q1);
-            }
-            if (RAG && nvl < 8) {
-                // the row's last octet is partial (nvl = 2, 4 or 6 for even
-                // X): the voxels past the end repeat the last one
-                const uint32_t e = nvl <= 2 ? v[3] : (nvl <= 4 ? v[5] : v[7]);
+                if (PART && nvl < 8) {
+                    const uint32_t e = nvl <= 2 ? v[3] : (nvl <= 4 ? v[5] : v[7]);
 #pragma unroll
-                for (int k = 4; k < 12; ++k)
-                    if (k >= 2 + nvl) v[k] = e;
+                    for (int k = 4; k < 12; ++k)
+                        if (k >= 2 + nvl) v[k] = e;
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) p[j] = v[j] + v[j + 4] + 4u * (v[j + 1] + v[j + 3]) + 6u * v[j + 2];
             }
             // this warp is done with the stage
             __syncwarp();
             if (lane == 0) mbar_arrive(S.empty + ST);
-            // x pass, then the z pass over planes k-4 .. k in gather form; the
+            // the z pass over planes k-4 .. k in gather form; the
             // 2048 enters with the outer pair so that s = sum >> 12 rounds
             // half up
             uint32_t s[8];
     #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const uint32_t p = v[j] + v[j + 4] + 4u * (v[j + 1] + v[j + 3]) + 6u * v[j + 2];
                 const uint32_t A = pr[(ST + 1) % FS_S][j], B = pr[(ST + 2) % FS_S][j];
                 const uint32_t C = pr[(ST + 3) % FS_S][j], D = pr[(ST + 4) % FS_S][j];
-                s[j] = (A + p + 2048u + 4u * (B + D) + 6u * C) >> 12;
-                pr[ST][j] = p;
+                s[j] = (A + p[j] + 2048u + 4u * (B + D) + 6u * C) >> 12;
+                pr[ST][j] = p[j];
             }
             if (k >= 4) {
-                if (RAG) {
+                if (PART) {
 #pragma unroll
                     for (int j = 2; j < 8; ++j)
                         if (j >= nvl) s[j] = 0u;  // not emitted (and below any t*)
@@ -1345,16 +1358,16 @@ __device__ __forceinline__ void smooth_rows_tile(const VolDev &V, uint32_t ix, u
                         // rows start 4-byte aligned only; the pairs past the end stay unwritten
 #pragma unroll
                         for (int j = 0; j < 8; j += 2)
-                            if (j < nvl) *reinterpret_cast<uint32_t *>(op + j) = s[j] | (s[j + 1] << 16);
+                            if (!PART || j < nvl) *reinterpret_cast<uint32_t *>(op + j) = s[j] | (s[j + 1] << 16);
                     }
                     if (fast) {
     #pragma unroll
                         for (int j = 0; j < 8; ++j)
-                            if (!RAG || j < nvl) atomicAdd(hc + s[j], 1u);
+                            if (!PART || j < nvl) atomicAdd(hc + s[j], 1u);
                     } else {
     #pragma unroll
                         for (int j = 0; j < 8; ++j) {
-                            if (RAG && j >= nvl) continue;
+                            if (PART && j >= nvl) continue;
                             const uint32_t u = min(s[j], 65535u);  // (always true for exact sums)
                             if (u < (uint32_t)HIST_LOW) {
                                 atomicAdd(hc + u, 1u);
@@ -1440,8 +1453,9 @@ __global__ void __launch_bounds__(FS_NT, 1) k_smooth_rows(const BatchHdr *__rest
         const int z0 = (int)(iz * V.fs_tz);
         const int z1 = min(z0 + (int)V.fs_tz, (int)V.Z);
         if (V.fs_rag) {
-            if (V.fs_hx) smooth_rows_tile<FS_RT, 1, 1>(V, ix, iy, z0, z1, ring, sh, S);
-            else smooth_rows_tile<0, 0, 1>(V, ix, iy, z0, z1, ring, sh, S);
+            if (!V.fs_hx) smooth_rows_tile<0, 0, 2>(V, ix, iy, z0, z1, ring, sh, S);
+            else if (ix + 1 < V.fs_ntx) smooth_rows_tile<FS_RT, 1, 1>(V, ix, iy, z0, z1, ring, sh, S);
+            else smooth_rows_tile<FS_RT, 1, 2>(V, ix, iy, z0, z1, ring, sh, S);
         } else if (V.fs_rt == (uint32_t)FS_RT) {
             if (V.fs_hx) smooth_rows_tile<FS_RT, 1, 0>(V, ix, iy, z0, z1, ring, sh, S);
             else smooth_rows_tile<FS_RT, 0, 0>(V, ix, iy, z0, z1, ring, sh, S);
@@ -1572,6 +1586,16 @@ __global__ void __launch_bounds__(ROW_TILE) k_threshold_runs(const BatchHdr *__r
                     if (vec) {
                         for (uint32_t o = 0; o < nv; o += 8u)
                             bits |= octet_bits(__ldcs(reinterpret_cast<const uint4 *>(src + xb + o)), t) << o;
+                    } else if (nv == 32u) {
+                        // all 16 pairs in flight at once (one at a time, each
+                        // load waited for the one before: 1795 against
+                        // XXX us for 5530 x 5530 x 80)
+                        uint32_t pr[16];
+#pragma unroll
+                        for (int o = 0; o < 16; ++o) pr[o] = __ldcs(reinterpret_cast<const unsigned int *>(src + xb + 2 * o));
+#pragma unroll
+                        for (int o = 0; o < 16; ++o)
+                            bits |= (((pr[o] & 0xFFFFu) > t ? 1u : 0u) | ((pr[o] >> 16) > t ? 2u : 0u)) << (2 * o);
                     } else {
                         for (uint32_t o = 0; o < nv; o += 2u) {
                             const uint32_t pr = __ldcs(reinterpret_cast<const unsigned int *>(src + xb + o));
@@ -1685,15 +1709,28 @@ __global__ void __launch_bounds__(ROW_TILE) k_threshold_runs(const BatchHdr *__r
                     }
                 }
             } else {
-                for (uint32_t xb = 0; xb < X; xb += 32) {
-                    const uint32_t x = xb + (uint32_t)lane;
-                    const bool on = x < X && __ldcs(src + x) > t;
-                    const uint32_t word = __ballot_sync(FULL, on);
-                    if (lane == 0) {
-                        dst[xb >> 5] = word;
-                        cnt += __popc(word & ~((word << 1) | carry));
+                // eight words' loads in flight before the first ballot
+                for (uint32_t xb0 = 0; xb0 < X; xb0 += 256) {
+                    uint32_t v[8];
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        const uint32_t x = xb0 + 32u * c + (uint32_t)lane;
+                        v[c] = x < X ? __ldcs(src + x) : 0u;
                     }
-                    carry = word >> 31;
+                    uint32_t mine = 0;  // lane c: word c of the eight
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        const uint32_t word = __ballot_sync(FULL, v[c] > t);
+                        if (lane == c) mine = word;
+                    }
+                    // run starts across the words, the first from the eight before
+                    const uint32_t prev = __shfl_up_sync(FULL, mine, 1);
+                    const uint32_t left = lane == 0 ? carry : prev >> 31;
+                    if (lane < 8 && xb0 + 32u * lane < X) {
+                        dst[(xb0 >> 5) + lane] = mine;
+                        cnt += __popc(mine & ~((mine << 1) | left));
+                    }
+                    carry = __shfl_sync(FULL, mine, 7) >> 31;
                 }
             }
 #pragma unroll
