@@ -59,7 +59,7 @@ struct VolDev {
     seg_cell_features *feat;  // k_cap cells output
     uint32_t *stat;           // ST_WORDS words
     uint32_t *hist;           // 65536 uint32 bins
-    uint16_t *smooth;         // [Z][Y][X] smoothed voxels (pass 1 -> threshold pass)
+    uint16_t *smooth;         // [Z][Y][sm_pitch] smoothed voxels (pass 1 -> threshold pass)
     uint16_t *wmax;           // rows x W: largest smoothed value of each mask word (k_smooth_rows
                               // volumes with X % 32 == 0 or X > 512; else null)
     uint32_t *mask;           // rows x W words, bit b of word w is x = 32w + b
@@ -73,6 +73,7 @@ struct VolDev {
     uint64_t k_cap;
     uint64_t r_cap;
     uint32_t X, Y, Z, W;      // W = words per mask row
+    uint32_t sm_pitch;        // voxels per row of smooth: X, or X rounded up to 8 (voxels past X are 0)
     uint32_t rows;            // Y * Z
     uint32_t min_volume;
     uint32_t union_limit;     // retries before a union gives up (ERR_UNION)

@@ -499,22 +499,22 @@ template <bool STORE>
 struct HistEmit {
     uint32_t *sh;
     uint32_t *gh;
-    uint16_t *sm;       // smoothed volume (STORE only)
-    uint32_t X, Y;
+    uint16_t *sm;       // smoothed volume (STORE only), rows of `pitch` voxels
+    uint32_t X, Y, pitch;
     uint32_t valid;     // bit j: voxel j of the octet is inside the volume
     uint32_t copy;      // word offset of this half-warp's copy of the low levels
     uint16_t *row;      // &sm[y * X + xb] at z = 0
     size_t zstride;     // voxels per z-plane
-    bool vec;           // all 8 inside and 16-byte aligned
+    bool vec;           // the row holds all 8, 16-byte aligned
     __device__ __forceinline__ void bind(int xb, int y) {
         valid = 0;
         if ((uint32_t)y < Y)
             for (int j = 0; j < 8; ++j) valid |= ((uint32_t)(xb + j) < X ? 1u : 0u) << j;
         copy = (threadIdx.x & 16u) ? (uint32_t)HIST_COPY1 : 0u;
         if (STORE) {
-            zstride = (size_t)X * Y;
-            row = sm + ((size_t)(valid ? (uint32_t)y : 0u) * X + (uint32_t)xb);
-            vec = valid == 0xFFu && (X & 7u) == 0u;
+            zstride = (size_t)pitch * Y;
+            row = sm + ((size_t)(valid ? (uint32_t)y : 0u) * pitch + (uint32_t)xb);
+            vec = valid != 0u && (pitch & 7u) == 0u;  // the row holds the whole octet
         }
     }
     __device__ __forceinline__ void operator()(int z, bool live, const uint32_t *s) {
@@ -534,8 +534,11 @@ struct HistEmit {
         if (STORE) {
             uint16_t *p = row + (size_t)(uint32_t)z * zstride;
             if (vec) {
+                uint32_t o[8];  // voxels past the volume are 0
+#pragma unroll
+                for (int j = 0; j < 8; ++j) o[j] = valid & (1u << j) ? s[j] : 0u;
                 *reinterpret_cast<uint4 *>(p) =
-                    make_uint4(s[0] | (s[1] << 16), s[2] | (s[3] << 16), s[4] | (s[5] << 16), s[6] | (s[7] << 16));
+                    make_uint4(o[0] | (o[1] << 16), o[2] | (o[3] << 16), o[4] | (o[5] << 16), o[6] | (o[7] << 16));
             } else {
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
@@ -978,7 +981,7 @@ __global__ void __launch_bounds__(8 * TY, 1) k_smooth_hist(const BatchHdr *__res
         const uint32_t iy = rest % V.nty, iz = rest / V.nty;
         const int z0 = (int)iz * tz;
         const int z1 = min(z0 + tz, (int)V.Z);
-        HistEmit<true> e{sh, V.hist, V.smooth, V.X, V.Y, 0u, 0u, nullptr, 0, false};
+        HistEmit<true> e{sh, V.hist, V.smooth, V.X, V.Y, V.sm_pitch, 0u, 0u, nullptr, 0, false};
         smooth_tile<TY>(V.raw, V.X, V.Y, V.Z, (int)ix * TILE_X, (int)iy * TY, z0, z1, spx, R, e);
     }
     flush_hist<T::NT>(h->vol[v], sh);
@@ -1178,6 +1181,15 @@ __device__ __forceinline__ void smooth_rows_tile(const VolDev &V, uint32_t ix, u
     const uint32_t plane = (uint32_t)X * (uint32_t)Y;  // < 2^32 (X Y Z < 2^32)
     const int n = z1 - z0 + 4;
     const uint32_t ring0 = smem_addr(ring);
+    // ragged rows of x-tiled volumes are staged a row per warp, consecutive
+    // lanes on consecutive 4-byte words (chunk by chunk, each copy
+    // instruction would touch four times the lines); words before or past
+    // the row are left out
+    constexpr bool BYROW = RAG != 0 && RTC != 0;
+    constexpr int BW = BYROW ? (4 * (RTC + 2 * HXC) + 31) / 32 : 1;  // copies per lane
+    const int brow = tid >> 5;
+    const uint32_t bsrc = BYROW ? (uint32_t)min(max(y0 - 2 + brow, 0), Y - 1) * (uint32_t)X : 0u;
+    const int bx = x0 - 8 * HXC + 2 * lane;  // this lane's first voxel pair
     // Tiles run through the ring in whole rounds of FS_S planes (a tile's
     // planes padded with planes that only keep the barriers' phases in step),
     // so that the stage of every plane is a compile-time constant; `par` is
@@ -1191,9 +1203,20 @@ __device__ __forceinline__ void smooth_rows_tile(const VolDev &V, uint32_t ix, u
         const bool ok = g0 + (uint32_t)k < (uint32_t)FS_S || S.wait(S.empty + ST, fp ^ 1u, stat);
         if (ok && k < n) {
             const uint32_t zoff = plane * (uint32_t)min(max(z0 - 2 + k, 0), Z - 1);
+            if (BYROW) {
+                if (brow < TYF + 4) {
+#pragma unroll
+                    for (int k = 0; k < BW; ++k) {
+                        const int x = bx + 64 * k;
+                        if (32 * k + lane < 4 * RC && x >= 0 && x < X)
+                            cp_async4(ring0 + ST * FS_STAGE + brow * RB + 4 * lane + 128 * k,
+                                      reinterpret_cast<uintptr_t>(raw + (bsrc + zoff + (uint32_t)x)), 4u);
+                    }
+                }
+            }
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-                if (!cok[u]) continue;
+                if (BYROW || !cok[u]) continue;
                 if (!RAG) {
                     cp_async16(ring0 + ST * FS_STAGE + cdst[u], reinterpret_cast<uintptr_t>(raw + (csrc[u] + zoff)));
                 } else {
@@ -1217,7 +1240,8 @@ __device__ __forceinline__ void smooth_rows_tile(const VolDev &V, uint32_t ix, u
     for (int i = 0; i < FS_S; ++i)
 #pragma unroll
         for (int j = 0; j < 8; ++j) pr[i][j] = 0u;
-    const uint32_t orow = (uint32_t)(y0 + tyc) * (uint32_t)X + (uint32_t)(x0 + 8 * q);
+    const uint32_t pitch = RAG ? V.sm_pitch : (uint32_t)X, oplane = RAG ? pitch * (uint32_t)Y : plane;
+    const uint32_t orow = (uint32_t)(y0 + tyc) * pitch + (uint32_t)(x0 + 8 * q);
     uint32_t *hc = sh + ((threadIdx.x & 16u) ? (uint32_t)HIST_COPY1 : 0u);
     // plane k from stage ST (full phase fp): nothing but the barriers for
     // the padding planes k >= n
@@ -1350,8 +1374,8 @@ __device__ __forceinline__ void smooth_rows_tile(const VolDev &V, uint32_t ix, u
                         wmax[(uint32_t)((z0 + k - 4) * Y + y0 + ty) * W + (uint32_t)((x0 + 8 * q) >> 5)] = (uint16_t)wm;
                 }
                 if (emit_ok) {
-                    uint16_t *op = osm + (orow + plane * (uint32_t)(z0 + k - 4));
-                    if (!RAG) {
+                    uint16_t *op = osm + (orow + oplane * (uint32_t)(z0 + k - 4));
+                    if (!RAG || (pitch & 7u) == 0u) {
                         *reinterpret_cast<uint4 *>(op) =
                             make_uint4(s[0] | (s[1] << 16), s[2] | (s[3] << 16), s[4] | (s[5] << 16), s[6] | (s[7] << 16));
                     } else {
@@ -1495,8 +1519,8 @@ __global__ void __launch_bounds__(ROW_TILE) k_threshold_runs(const BatchHdr *__r
         const uint32_t lt = rt - V.rt_base;
         const uint32_t row0 = lt * h->row_tile;
         const uint32_t nrows = min(h->row_tile, V.rows - row0);
-        const uint32_t X = V.X, W = V.W, t = V.stat[ST_THRESH];
-        const bool vec = (X & 7u) == 0u;
+        const uint32_t X = V.X, W = V.W, t = V.stat[ST_THRESH], P = V.sm_pitch;
+        const bool vec = (P & 7u) == 0u;  // (voxels of a row past X are 0: never above t)
         uint32_t wtot = 0;
         const uint16_t *wmax = V.wmax;
         if (wmax && (X & 255u) == 0u && W <= 256u && ((W >> 3) & ((W >> 3) - 1u)) == 0u) {
@@ -1523,7 +1547,7 @@ __global__ void __launch_bounds__(ROW_TILE) k_threshold_runs(const BatchHdr *__r
                 uint32_t word[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) word[i] = 0u;
-                const uint16_t *src = V.smooth + (size_t)(row0 + rr) * X + 32u * lw;
+                const uint16_t *src = V.smooth + (size_t)(row0 + rr) * P + 32u * lw;
                 for (uint32_t a = act; a; a &= a - 1u) {
                     const int i = __ffs(a) - 1;
                     const uint4 *p = reinterpret_cast<const uint4 *>(src + 32 * i);
@@ -1563,9 +1587,9 @@ __global__ void __launch_bounds__(ROW_TILE) k_threshold_runs(const BatchHdr *__r
             // 16-byte loop below does not take (X % 8 != 0, or X > 512): a lane owns
             // 8 consecutive mask words (lanes past the row's words hold none),
             // a row is seg lanes (the power of two >= W / 8).  Each word
-            // above t* is read as octets (16-byte aligned rows, X % 8 == 0)
-            // or as voxel pairs (rows of an even X start 4-byte aligned);
-            // the last word of a row stops at X.
+            // above t* is read as octets (smoothed rows of whole octets) or as
+            // voxel pairs (rows of an even X start 4-byte aligned); the last
+            // word of a row stops at X.
             uint32_t seg = 1u;
             while (seg * 8u < W) seg <<= 1;
             const uint32_t rows_pw = 32u / seg;
@@ -1574,35 +1598,42 @@ __global__ void __launch_bounds__(ROW_TILE) k_threshold_runs(const BatchHdr *__r
                 const uint32_t rr = rb + lrow;
                 const bool live = rr < nrows;
                 const uint16_t *mp = wmax + (size_t)(row0 + rr) * W;
-                const uint16_t *src = V.smooth + (size_t)(row0 + rr) * X;
-                uint32_t word[8];
+                const uint16_t *src = V.smooth + (size_t)(row0 + rr) * P;
+                uint32_t act = 0;  // bit i: word lw + i has a voxel above t*
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    word[i] = 0u;
                     const uint32_t w = lw + (uint32_t)i;
-                    if (!live || w >= W || mp[w] <= t) continue;
-                    const uint32_t xb = 32u * w, nv = min(32u, X - xb);  // voxels of word w
+                    const uint32_t m = live && w < W ? mp[w] : 0u;
+                    act |= (m > t ? 1u : 0u) << i;
+                }
+                uint32_t word[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) word[i] = 0u;
+                for (uint32_t a = act; a; a &= a - 1u) {
+                    const int i = __ffs(a) - 1;
+                    const uint32_t xb = 32u * (lw + (uint32_t)i), nv = min(32u, X - xb);  // voxels of the word
                     uint32_t bits = 0u;
+                    // all loads of a word in flight at once
                     if (vec) {
-                        for (uint32_t o = 0; o < nv; o += 8u)
-                            bits |= octet_bits(__ldcs(reinterpret_cast<const uint4 *>(src + xb + o)), t) << o;
-                    } else if (nv == 32u) {
-                        // all 16 pairs in flight at once (one at a time, each
-                        // load waited for the one before: 1795 against
-                        // XXX us for 5530 x 5530 x 80)
+                        uint4 q4[4];
+#pragma unroll
+                        for (int o = 0; o < 4; ++o)
+                            q4[o] = 8u * o < nv ? __ldcs(reinterpret_cast<const uint4 *>(src + xb + 8 * o))
+                                                : make_uint4(0, 0, 0, 0);
+#pragma unroll
+                        for (int o = 0; o < 4; ++o) bits |= octet_bits(q4[o], t) << (8 * o);
+                    } else {
                         uint32_t pr[16];
 #pragma unroll
-                        for (int o = 0; o < 16; ++o) pr[o] = __ldcs(reinterpret_cast<const unsigned int *>(src + xb + 2 * o));
+                        for (int o = 0; o < 16; ++o)
+                            pr[o] = 2u * o < nv ? __ldcs(reinterpret_cast<const unsigned int *>(src + xb + 2 * o)) : 0u;
 #pragma unroll
                         for (int o = 0; o < 16; ++o)
                             bits |= (((pr[o] & 0xFFFFu) > t ? 1u : 0u) | ((pr[o] >> 16) > t ? 2u : 0u)) << (2 * o);
-                    } else {
-                        for (uint32_t o = 0; o < nv; o += 2u) {
-                            const uint32_t pr = __ldcs(reinterpret_cast<const unsigned int *>(src + xb + o));
-                            bits |= (((pr & 0xFFFFu) > t ? 1u : 0u) | ((pr >> 16) > t ? 2u : 0u)) << o;
-                        }
                     }
-                    word[i] = bits;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        if (k == i) word[k] = bits;
                 }
                 uint32_t left = __shfl_up_sync(FULL, word[7], 1) >> 31;
                 if (lw == 0u) left = 0u;
@@ -1637,7 +1668,7 @@ __global__ void __launch_bounds__(ROW_TILE) k_threshold_runs(const BatchHdr *__r
                     for (int c = 0; c < 2; ++c) {
                         const uint32_t x = 256u * c + 8u * (uint32_t)lane;
                         q4[k][c] = (rr < nrows && x < X)
-                                       ? __ldcs(reinterpret_cast<const uint4 *>(V.smooth + (size_t)(row0 + rr) * X + x))
+                                       ? __ldcs(reinterpret_cast<const uint4 *>(V.smooth + (size_t)(row0 + rr) * P + x))
                                        : make_uint4(0, 0, 0, 0);
                     }
                 }
@@ -1675,7 +1706,7 @@ __global__ void __launch_bounds__(ROW_TILE) k_threshold_runs(const BatchHdr *__r
         } else
         for (uint32_t rr = warp; rr < nrows; rr += WARPS) {
             const uint32_t row = row0 + rr;
-            const uint16_t *src = V.smooth + (size_t)row * X;
+            const uint16_t *src = V.smooth + (size_t)row * P;
             uint32_t *dst = V.mask + (size_t)row * W;
             uint32_t carry = 0, cnt = 0;
             if (vec) {
@@ -4457,7 +4488,7 @@ __global__ void __launch_bounds__(8 * TY, 1) k_smooth_hist_noalloc(const __grid_
         const uint32_t iy = rest % V.nty, iz = rest / V.nty;
         const int z0 = (int)iz * tz;
         const int z1 = min(z0 + tz, (int)V.Z);
-        HistEmit<false> e{sh, V.hist, nullptr, V.X, V.Y, 0u, 0u, nullptr, 0, false};
+        HistEmit<false> e{sh, V.hist, nullptr, V.X, V.Y, 0u, 0u, 0u, nullptr, 0, false};
         smooth_tile<TY>(V.raw, V.X, V.Y, V.Z, (int)ix * TILE_X, (int)iy * TY, z0, z1, spx, R, e);
     }
     flush_hist<T::NT>(V, sh);

@@ -510,7 +510,20 @@ void build_header(seg_ctx *ctx, Batch &b) {
             }
             V.hist = reinterpret_cast<uint32_t *>(sp); sp += al(4ull * HIST_BINS);
             V.smooth = reinterpret_cast<uint16_t *>(sp); sp += al(2ull * g.n);
-            if (r->smoothed(c)) V.smooth = r->smoothed(c);
+            V.sm_pitch = g.X;
+            if (r->smoothed(c)) {
+                V.smooth = r->smoothed(c);
+            } else if (g.X % 8u != 0u) {
+                // rows of X % 8 != 0 voxels go into the label image, unused
+                // until the label kernel, with rows padded to whole octets
+                // (2 bytes a voxel of at most 2 X), so that the smoothing
+                // stores and the threshold loads 16 bytes at a time
+                const uint32_t p = (g.X + 7u) / 8u * 8u;
+                if (p <= 2u * g.X && (uint64_t)p * g.rows < (1ull << 32)) {
+                    V.smooth = reinterpret_cast<uint16_t *>(V.labels);
+                    V.sm_pitch = p;
+                }
+            }
             V.wmax = reinterpret_cast<uint16_t *>(sp); sp += al(2ull * g.rows * g.W);
             V.mask = reinterpret_cast<uint32_t *>(sp); sp += al(4ull * g.rows * g.W);
             V.rowoff = reinterpret_cast<uint32_t *>(sp); sp += al(4ull * (g.rows + 1));
