@@ -273,6 +273,11 @@ cudaError_t launch_label_runs_write(const uint32_t *labels, uint32_t X, uint32_t
                                     const uint32_t *tiles, const uint32_t *total, uint64_t cap, seg_label_run *out,
                                     seg_label_run *mapped, int sms, cudaStream_t s);
 
+// z-chunk for `columns` tile columns of Z planes on `blocks` blocks that take
+// equal shares of the tiles: the one whose fullest block smooths the fewest
+// planes, the four halo planes of each tile counted.
+uint32_t hist_tile_z(uint64_t columns, uint32_t Z, uint32_t blocks);
+
 // Histogram-kernel shared memory per block for a tile height.
 size_t hist_smem_bytes(int tile_y);
 // k_smooth_rows: threads per block, octets per tile row at most, and the
