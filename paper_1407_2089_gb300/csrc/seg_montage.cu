@@ -11,10 +11,11 @@
 //     zero outside its box, so no bounds test per product), and each thread
 //     takes shifts, summing the products over the sub-box from shared
 //     memory;
-//   * Sa, Saa (tile a) and Sb, Sbb (tile b) from the x-range sums of every
-//     row (k_reg_rows), their prefixes along y per x-range and plane
-//     (k_reg_q), then per shift a sum over the planes of its box
-//     (k_reg_box), because the shared box varies only at its faces.
+//   * Sa, Saa (tile a) and Sb, Sbb (tile b) from the sums of every plane over
+//     each shift's x- and y-range (k_reg_plane), because the shared box varies
+//     only at its faces, then per shift a sum over the planes of its box
+//     (k_reg_box).
+// Every kernel takes all pairs of a group in one launch.
 // The host then forms the Pearson correlation in 128-bit integers and
 // binary64, picks the first best shift in z, y, x order, builds the maximum
 // spanning tree (Kruskal) and sums the shifts from the root.
@@ -32,8 +33,12 @@
 
 namespace {
 
-constexpr int RC_TX = 32, RC_TY = 8, RC_TZ = 8;  // tile-a sub-box of a k_reg_corr block
+constexpr int RC_TX = 32, RC_TY = 16, RC_TZ = 16;  // tile-a sub-box of a k_reg_corr block
 constexpr int RC_THREADS = 256;
+static_assert(RC_TY >= RC_THREADS / 32 && RC_TX == 32, "staging by row per warp");
+// row pitch of the staged tile-b region: an odd number of 32-bit words, so that
+// lanes on consecutive rows read distinct banks
+__host__ __device__ constexpr int rc_pitch(int rx) { return 2 * (((RC_TX + 2 * rx + 1) / 2) | 1); }
 
 // Half-open range [lo, hi) of one axis.
 struct Range {
@@ -47,66 +52,165 @@ __host__ __device__ inline Range shared_range(int d, int D, int side) {
     return Range{-d > 0 ? -d : 0, D - d < D ? D - d : D};
 }
 
-// Sab for every shift: block = sub-box (RC_TX x RC_TY x RC_TZ) of tile a's
-// search region U (in a's coordinates).  Shift index
+// One overlapping pair on the device: tile b's origin in tile a's frame, the
+// search region of each side (0: a, 1: b) in that tile's frame, and where the
+// plane sums of each side start.
+struct RegPair {
+    const uint16_t *tile[2];
+    int3 d0;
+    int3 u0[2], u1[2];
+    size_t planes[2];
+};
+
+// Sab for every shift: block (x, y) = sub-box x (RC_TX x RC_TY x RC_TZ) of the
+// search region U of tile a of pair y (in a's coordinates).  Shift index
 // si = ((sz + rz) SY + (sy + ry)) SX + (sx + rx).  Thread (g, c) takes the
 // (y, z)-shift g = (sy, sz) for every x-shift (KX = 2 RX + 1 of them) over
 // the sub-box rows c, c + C, ...: along a row the x-shifts need b values
 // x + 2 RX - k, so a register window of KX b values slides with x and every
-// product costs one multiply-add.  The threads' sums meet in shared memory
-// and go out with one atomic per (block, shift).
+// product costs one multiply-add.  Products are added in 32 bits over as many
+// rows as the sub-box's largest values allow (32 rows at 2000 x 2000), then
+// moved to 64-bit sums; only where one row could overflow are the sums 64-bit
+// throughout (three instructions per product instead of one).  Bound by
+// instruction issue (one multiply-add per product, a third more for staging
+// and unpacking): 1.93 ms for the 20.5 G products of 3 x 3 tiles of 1024 x 1024
+// x 64 with a tenth of overlap and radius 4, 4, 1, where 64-bit sums over 8 x 8
+// rows took 3.2 ms; 8 x 16 rows take 2.1 ms.  The threads' sums meet in shared memory and go out with one atomic
+// per (block, shift).
 template <int RX>
-__global__ void __launch_bounds__(RC_THREADS) k_reg_corr(const uint16_t *__restrict__ A, const uint16_t *__restrict__ B,
-                                                         int X, int Y, int Z, int3 u0, int3 u1, int3 d0, int ry,
-                                                         int rz, unsigned long long *__restrict__ sab) {
+__global__ void __launch_bounds__(RC_THREADS) k_reg_corr(const RegPair *__restrict__ pairs, int X, int Y, int Z, int ry,
+                                                         int rz, unsigned long long *__restrict__ sums, size_t per) {
     constexpr int KX = 2 * RX + 1;
-    constexpr int BX = RC_TX + 2 * RX;
+    constexpr int BX = RC_TX + 2 * RX, BP = rc_pitch(RX);
     extern __shared__ __align__(16) unsigned long long rsm64[];
+    __shared__ uint32_t smax[2];
+    const RegPair &P = pairs[blockIdx.y];
+    const uint16_t *__restrict__ A = P.tile[0], *__restrict__ B = P.tile[1];
+    const int3 u0 = P.u0[0], u1 = P.u1[0], d0 = P.d0;
+    unsigned long long *sab = sums + per * blockIdx.y;
     const int BY = RC_TY + 2 * ry, BZ = RC_TZ + 2 * rz, SY = 2 * ry + 1, G = SY * (2 * rz + 1);
     unsigned long long *red = rsm64;                                      // [G][KX]
-    uint16_t *As = reinterpret_cast<uint16_t *>(rsm64 + (size_t)G * KX);  // [RC_TZ][RC_TY][RC_TX]
-    uint16_t *Bs = As + RC_TX * RC_TY * RC_TZ;                            // [BZ][BY][BX]
+    uint16_t *As = reinterpret_cast<uint16_t *>(rsm64 + ((size_t)G * KX + 1) / 2 * 2);  // [RC_TZ][RC_TY][RC_TX]
+    uint16_t *Bs = As + RC_TX * RC_TY * RC_TZ;                            // [BZ][BY][BP]
+    if (u1.x <= u0.x || u1.y <= u0.y || u1.z <= u0.z) return;
     const int nbx = (u1.x - u0.x + RC_TX - 1) / RC_TX, nby = (u1.y - u0.y + RC_TY - 1) / RC_TY;
+    const int nbz = (u1.z - u0.z + RC_TZ - 1) / RC_TZ;
     const int bi = (int)blockIdx.x;
+    if ((long long)bi >= (long long)nbx * nby * nbz) return;
     const int ax0 = u0.x + (bi % nbx) * RC_TX, ay0 = u0.y + ((bi / nbx) % nby) * RC_TY;
     const int az0 = u0.z + (bi / (nbx * nby)) * RC_TZ;
+    if (threadIdx.x < 2) smax[threadIdx.x] = 0u;
     for (int i = threadIdx.x; i < G * KX; i += RC_THREADS) red[i] = 0ull;
-    for (int i = threadIdx.x; i < RC_TX * RC_TY * RC_TZ; i += RC_THREADS) {
-        const int x = ax0 + i % RC_TX, y = ay0 + (i / RC_TX) % RC_TY, z = az0 + i / (RC_TX * RC_TY);
-        As[i] = (x < u1.x && y < u1.y && z < u1.z) ? A[((size_t)z * Y + y) * X + x] : (uint16_t)0;
+    __syncthreads();
+    // a row per warp, four rows' loads in flight
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int WARPS = RC_THREADS / 32, RB = 4;
+    uint32_t ma = 0, mb = 0;
+    for (int r0 = warp; r0 < RC_TY * RC_TZ; r0 += WARPS * RB) {
+        uint32_t v[RB];
+#pragma unroll
+        for (int k = 0; k < RB; ++k) {
+            const int row = r0 + k * WARPS, x = ax0 + lane, y = ay0 + row % RC_TY, z = az0 + row / RC_TY;
+            v[k] = row < RC_TY * RC_TZ && x < u1.x && y < u1.y && z < u1.z ? A[((size_t)z * Y + y) * X + x] : 0u;
+        }
+#pragma unroll
+        for (int k = 0; k < RB; ++k) {
+            const int row = r0 + k * WARPS;
+            if (row < RC_TY * RC_TZ) As[row * RC_TX + lane] = (uint16_t)v[k];
+            ma = max(ma, v[k]);
+        }
     }
     // b coordinates of a's sub-box under every shift: a - d0 - s
     const int bx0 = ax0 - d0.x - RX, by0 = ay0 - d0.y - ry, bz0 = az0 - d0.z - rz;
-    for (int i = threadIdx.x; i < BX * BY * BZ; i += RC_THREADS) {
-        const int x = bx0 + i % BX, y = by0 + (i / BX) % BY, z = bz0 + i / (BX * BY);
-        Bs[i] = (x >= 0 && x < X && y >= 0 && y < Y && z >= 0 && z < Z) ? B[((size_t)z * Y + y) * X + x]
-                                                                       : (uint16_t)0;
+    const int xa = bx0 + lane, xb = xa + 32;  // (BX <= 56)
+    const bool ina = xa >= 0 && xa < X, inb = xb >= 0 && xb < X && lane + 32 < BX;
+    // row = warp, warp + WARPS, ... as (ty, tz), stepped without divisions (BY >= WARPS)
+    int ty = warp, tz = 0;
+    for (int r0 = warp; r0 < BY * BZ; r0 += WARPS * RB) {
+        uint32_t v[RB], w[RB];
+#pragma unroll
+        for (int k = 0; k < RB; ++k) {
+            const int y = by0 + ty, z = bz0 + tz;
+            const bool in = tz < BZ && y >= 0 && y < Y && z >= 0 && z < Z;
+            const uint16_t *b = B + (in ? ((size_t)z * Y + y) * X : 0);
+            v[k] = in && ina ? b[xa] : 0u;
+            w[k] = in && inb ? b[xb] : 0u;
+            ty += WARPS;
+            if (ty >= BY) {
+                ty -= BY;
+                ++tz;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < RB; ++k) {
+            const int row = r0 + k * WARPS;
+            if (row < BY * BZ) {
+                Bs[row * BP + lane] = (uint16_t)v[k];
+                if (lane + 32 < BX) Bs[row * BP + lane + 32] = (uint16_t)w[k];
+            }
+            mb = max(mb, max(v[k], w[k]));
+        }
+    }
+    ma = __reduce_max_sync(0xFFFFFFFFu, ma);
+    mb = __reduce_max_sync(0xFFFFFFFFu, mb);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&smax[0], ma);
+        atomicMax(&smax[1], mb);
     }
     __syncthreads();
     constexpr int ROWS = RC_TY * RC_TZ;
     const int C = G >= RC_THREADS ? 1 : min(ROWS, RC_THREADS / G);  // row chunks per shift group
+    // rows whose products sum to less than 2^32: each of the RC_TX products
+    // is at most smax[0] smax[1] (< 2^32)
+    const uint32_t most = smax[0] * smax[1];
+    const int fit = most ? (int)min(0xFFFFFFFFu / most / RC_TX, (uint32_t)ROWS) : ROWS;
+    // one row: acc[k] += a(x) b(x + 2 RX - k) over x
+    auto add_row = [&](int row, int sy, int sz, auto &acc) {
+        const int y = row % RC_TY, z = row / RC_TY;
+        const uint4 *ar = reinterpret_cast<const uint4 *>(As + row * RC_TX);
+        const uint32_t *br = reinterpret_cast<const uint32_t *>(Bs + ((z - sz + rz) * BY + (y - sy + ry)) * BP);
+        uint32_t win[KX + 1];  // b at x .. x + 2 RX (+ 1): win[(x + j) % (KX + 1)] holds b(x + j)
+#pragma unroll
+        for (int j = 0; j < RX; ++j) {
+            const uint32_t w = br[j];
+            win[2 * j] = w & 0xFFFFu;
+            win[2 * j + 1] = w >> 16;
+        }
+#pragma unroll
+        for (int x0 = 0; x0 < RC_TX; x0 += 8) {
+            const uint4 a4 = ar[x0 / 8];
+            const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w};
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const int x = x0 + 2 * h;
+                const uint32_t w = br[RX + x / 2];  // b at x + 2 RX, x + 2 RX + 1
+                win[(x + 2 * RX) % (KX + 1)] = w & 0xFFFFu;
+                win[(x + 2 * RX + 1) % (KX + 1)] = w >> 16;
+                const uint32_t al = aw[h] & 0xFFFFu, ah = aw[h] >> 16;
+#pragma unroll
+                for (int k = 0; k < KX; ++k) acc[k] += al * win[(x + 2 * RX - k) % (KX + 1)];
+#pragma unroll
+                for (int k = 0; k < KX; ++k) acc[k] += ah * win[(x + 1 + 2 * RX - k) % (KX + 1)];
+            }
+        }
+    };
     for (int w = threadIdx.x; w < G * C; w += RC_THREADS) {
         const int g = w % G, c = w / G;
         const int sy = g % SY - ry, sz = g / SY - rz;
         unsigned long long acc[KX];
 #pragma unroll
         for (int k = 0; k < KX; ++k) acc[k] = 0ull;
-        for (int row = c; row < ROWS; row += C) {
-            const int y = row % RC_TY, z = row / RC_TY;
-            const uint16_t *ar = As + row * RC_TX;
-            const uint16_t *br = Bs + ((z - sz + rz) * BY + (y - sy + ry)) * BX;
-            uint32_t win[KX];  // b at x .. x + 2 RX
+        if (fit > 0) {
+            for (int row = c; row < ROWS;) {
+                uint32_t part[KX];
 #pragma unroll
-            for (int j = 0; j < KX - 1; ++j) win[j + 1] = br[j];
+                for (int k = 0; k < KX; ++k) part[k] = 0u;
+                for (int n = 0; n < fit && row < ROWS; ++n, row += C) add_row(row, sy, sz, part);
 #pragma unroll
-            for (int x = 0; x < RC_TX; ++x) {
-#pragma unroll
-                for (int j = 0; j < KX - 1; ++j) win[j] = win[j + 1];
-                win[KX - 1] = br[x + 2 * RX];
-                const uint32_t a = ar[x];
-#pragma unroll
-                for (int k = 0; k < KX; ++k) acc[k] += (unsigned long long)(a * win[2 * RX - k]);
+                for (int k = 0; k < KX; ++k) acc[k] += part[k];
             }
+        } else {
+            for (int row = c; row < ROWS; row += C) add_row(row, sy, sz, acc);
         }
 #pragma unroll
         for (int k = 0; k < KX; ++k)
@@ -120,12 +224,11 @@ __global__ void __launch_bounds__(RC_THREADS) k_reg_corr(const uint16_t *__restr
 // Shared memory of k_reg_corr<RX>.
 size_t reg_corr_smem(int rx, int ry, int rz) {
     const size_t G = (size_t)(2 * ry + 1) * (2 * rz + 1), KX = 2 * rx + 1;
-    return 8 * G * KX + 2 * ((size_t)RC_TX * RC_TY * RC_TZ +
-                             (size_t)(RC_TX + 2 * rx) * (RC_TY + 2 * ry) * (RC_TZ + 2 * rz));
+    return 16 * ((G * KX + 1) / 2) + 2 * ((size_t)RC_TX * RC_TY * RC_TZ +
+                             (size_t)rc_pitch(rx) * (RC_TY + 2 * ry) * (RC_TZ + 2 * rz));
 }
 
-using RegCorrFn = void (*)(const uint16_t *, const uint16_t *, int, int, int, int3, int3, int3, int, int,
-                           unsigned long long *);
+using RegCorrFn = void (*)(const RegPair *, int, int, int, int, int, unsigned long long *, size_t);
 template <int... R>
 RegCorrFn reg_corr_fn(int rx, std::integer_sequence<int, R...>) {
     RegCorrFn f = nullptr;
@@ -133,139 +236,164 @@ RegCorrFn reg_corr_fn(int rx, std::integer_sequence<int, R...>) {
     return f;
 }
 
-// Per row (y, z) of the region U of one tile and x-shift sxi: the sums of v
-// and v^2 over the shift's x-range, R[sxi rows + row] with row =
-// (z - u0.z) UY + (y - u0.y).  One warp per row: the part of the row every
-// x-range shares (the core) is summed by all lanes and reduced; lane sxi then
-// adds its range's voxels outside the core (at most 2 rx of them).
-__global__ void k_reg_rows(const uint16_t *__restrict__ T, int X, int Y, int3 u0, int3 u1, int d0x, int rx, int side,
-                           unsigned long long *__restrict__ r1, unsigned long long *__restrict__ r2) {
-    const int UY = u1.y - u0.y, rows = UY * (u1.z - u0.z), SX = 2 * rx + 1;
+// Sums of v and v^2 over one plane of a side's region U for every x-range (one
+// per x-shift) and y-range (one per y-shift): p1, p2[((z - u0.z) SY + syi) SX +
+// sxi].  Block (z, 2 pair + side).  Ranges move monotonically with the shift:
+// all of them share a core [clo, chi) in x and in y, and outside it lie at most
+// 2 rx columns on either side.  The rows of the y-core add up in registers, the
+// x-core per lane and the outer columns one per lane, and are reduced once per
+// plane; only the at most 4 ry rows outside the y-core are reduced row by row
+// and added to the y-ranges that hold them.  Where the ranges share no core in
+// x the region is at most 2 rx columns wide (the overlap or the tile is
+// narrower than the window), and all of them count as left outer ones.  Bound
+// by reading the plane.
+constexpr int RP_THREADS = 256, RP_SY = 2 * SEG_REG_MAX_RXY + 1;
+constexpr int RP_COLS = 64;  // outer columns: 32 left, 32 right (2 rx <= 24 used)
+
+__global__ void __launch_bounds__(RP_THREADS) k_reg_plane(const RegPair *__restrict__ pairs, int X, int Y, int3 r,
+                                                          unsigned long long *__restrict__ p1,
+                                                          unsigned long long *__restrict__ p2) {
+    // sums of v and v^2: entry SY holds the y-core, entry syi the other rows
+    // of y-range syi; the x-core, and each outer column
+    __shared__ unsigned long long xc[2][RP_SY + 1], col[2][RP_SY + 1][RP_COLS];
+    const RegPair &P = pairs[blockIdx.y >> 1];
+    const int side = blockIdx.y & 1;
+    const int3 u0 = P.u0[side], u1 = P.u1[side], d0 = P.d0;
+    if (u1.x <= u0.x || u1.y <= u0.y || (int)blockIdx.x >= u1.z - u0.z) return;
+    const int SX = 2 * r.x + 1, SY = 2 * r.y + 1;
     const int lane = threadIdx.x & 31;
-    const Range first = shared_range(d0x - rx, X, side), last = shared_range(d0x + rx, X, side);
-    // ranges move monotonically with the shift: the core is [max lo, min hi)
-    const int clo = max(first.lo, last.lo), chi = min(first.hi, last.hi);
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < rows; row += nw) {
-        const int y = u0.y + row % UY, z = u0.z + row / UY;
-        const uint16_t *t = T + ((size_t)z * Y + y) * X;
-        unsigned long long a = 0, b = 0;
-        for (int x = clo + lane; x < chi; x += 32) {
-            const unsigned long long v = t[x];
-            a += v;
-            b += v * v;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
-            b += __shfl_xor_sync(0xFFFFFFFFu, b, o);
-        }
-        if (lane < SX) {
-            const Range q = shared_range(d0x + lane - rx, X, side);
-            if (clo >= chi) {  // no core: the whole range
-                a = b = 0;
-                for (int x = q.lo; x < q.hi; ++x) {
-                    const unsigned long long v = t[x];
-                    a += v;
-                    b += v * v;
-                }
-            } else if (q.lo >= q.hi) {
-                a = b = 0;
-            } else {
-                for (int x = q.lo; x < clo; ++x) {
-                    const unsigned long long v = t[x];
-                    a += v;
-                    b += v * v;
-                }
-                for (int x = chi; x < q.hi; ++x) {
-                    const unsigned long long v = t[x];
-                    a += v;
-                    b += v * v;
-                }
-            }
-            r1[(size_t)lane * rows + row] = a;
-            r2[(size_t)lane * rows + row] = b;
-        }
-    }
-}
-
-// For every x-shift and plane of U: prefix along y of the rows' sums over the
-// shift's x-range.  Q[(sxi (UZ) + z - u0.z) (UY + 1) + j].  One block per
-// (x-shift, plane): each thread sums a run of consecutive rows, a block scan
-// of the run totals gives each run's start, then the runs are written.
-constexpr int RQ_THREADS = 256;
-__global__ void __launch_bounds__(RQ_THREADS) k_reg_q(const unsigned long long *__restrict__ r1,
-                                                      const unsigned long long *__restrict__ r2, int3 u0, int3 u1,
-                                                      unsigned long long *__restrict__ q1,
-                                                      unsigned long long *__restrict__ q2) {
-    __shared__ unsigned long long t1[RQ_THREADS], t2[RQ_THREADS];
-    const int UY = u1.y - u0.y, UZ = u1.z - u0.z, rows = UY * UZ;
-    const int i = (int)blockIdx.x, sxi = i / UZ, zz = i % UZ;
-    const unsigned long long *s1 = r1 + (size_t)sxi * rows + (size_t)zz * UY;
-    const unsigned long long *s2 = r2 + (size_t)sxi * rows + (size_t)zz * UY;
-    const int per = (UY + RQ_THREADS - 1) / RQ_THREADS, j0 = threadIdx.x * per, j1 = min(j0 + per, UY);
-    unsigned long long a = 0, b = 0;
-    for (int j = j0; j < j1; ++j) {
-        a += s1[j];
-        b += s2[j];
-    }
-    t1[threadIdx.x] = a;
-    t2[threadIdx.x] = b;
+    for (int i = threadIdx.x; i < 2 * (RP_SY + 1); i += RP_THREADS) (&xc[0][0])[i] = 0ull;
+    for (int i = threadIdx.x; i < 2 * (RP_SY + 1) * RP_COLS; i += RP_THREADS) (&col[0][0][0])[i] = 0ull;
+    const Range xf = shared_range(d0.x - r.x, X, side), xl = shared_range(d0.x + r.x, X, side);
+    const Range yf = shared_range(d0.y - r.y, Y, side), yl = shared_range(d0.y + r.y, Y, side);
+    int clo = max(xf.lo, xl.lo), chi = min(xf.hi, xl.hi);
+    const int ylo = max(yf.lo, yl.lo), yhi = min(yf.hi, yl.hi);
+    if (clo >= chi) clo = chi = u1.x;  // no core: at most 4 rx columns, all left ones
+    // this lane's outer columns: u0.x + lane before clo, and chi + lane
+    const int xa = u0.x + lane, xr = chi + lane;
     __syncthreads();
-    // inclusive scan of the run totals (Hillis-Steele)
-    for (int o = 1; o < RQ_THREADS; o <<= 1) {
-        const unsigned long long x = threadIdx.x >= o ? t1[threadIdx.x - o] : 0ull;
-        const unsigned long long y = threadIdx.x >= o ? t2[threadIdx.x - o] : 0ull;
-        __syncthreads();
-        t1[threadIdx.x] += x;
-        t2[threadIdx.x] += y;
-        __syncthreads();
-    }
-    unsigned long long *o1 = q1 + (size_t)i * (UY + 1), *o2 = q2 + (size_t)i * (UY + 1);
-    a = t1[threadIdx.x] - a;  // exclusive start of this run
-    b = t2[threadIdx.x] - b;
-    if (threadIdx.x == 0) {
-        o1[0] = 0;
-        o2[0] = 0;
-    }
-    for (int j = j0; j < j1; ++j) {
-        a += s1[j];
-        b += s2[j];
-        o1[j + 1] = a;
-        o2[j + 1] = b;
-    }
-}
-
-// Per shift: the sums of v and v^2 over the tile's shared box; one warp per
-// shift, lanes over the planes of the box.
-__global__ void k_reg_box(const unsigned long long *__restrict__ q1, const unsigned long long *__restrict__ q2,
-                          int X, int Y, int Z, int3 u0, int3 u1, int3 d0, int3 r, int side,
-                          unsigned long long *__restrict__ s1, unsigned long long *__restrict__ s2) {
-    const int UY = u1.y - u0.y, UZ = u1.z - u0.z, lane = threadIdx.x & 31;
-    const int SX = 2 * r.x + 1, SY = 2 * r.y + 1, S = SX * SY * (2 * r.z + 1);
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int si = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; si < S; si += nw) {
-        const int sxi = si % SX, sy = (si / SX) % SY - r.y, sz = si / (SX * SY) - r.z;
-        const Range xr = shared_range(d0.x + sxi - r.x, X, side);
-        const Range yr = shared_range(d0.y + sy, Y, side), zr = shared_range(d0.z + sz, Z, side);
-        unsigned long long a = 0, b = 0;
-        if (xr.lo < xr.hi && yr.lo < yr.hi && zr.lo < zr.hi) {
-            for (int z = zr.lo + lane; z < zr.hi; z += 32) {
-                const size_t q = (size_t)(sxi * UZ + (z - u0.z)) * (UY + 1);
-                a += q1[q + (yr.hi - u0.y)] - q1[q + (yr.lo - u0.y)];
-                b += q2[q + (yr.hi - u0.y)] - q2[q + (yr.lo - u0.y)];
+    const uint16_t *plane = P.tile[side] + (size_t)(u0.z + (int)blockIdx.x) * X * Y;
+    unsigned long long a1 = 0, a2 = 0, l1 = 0, l2 = 0, h1 = 0, h2 = 0;  // y-core
+    constexpr int WARPS = RP_THREADS / 32, RB = 4;
+    const int warp = threadIdx.x >> 5;
+    // the y-core, RB rows' loads in flight
+    for (int y0 = ylo + warp; y0 < yhi; y0 += WARPS * RB) {
+        const uint16_t *t[RB];
+        bool on[RB];
+        uint32_t va[RB], vr[RB];
+#pragma unroll
+        for (int k = 0; k < RB; ++k) {
+            const int y = y0 + k * WARPS;
+            on[k] = y < yhi;
+            t[k] = plane + (size_t)(on[k] ? y : y0) * X;
+            va[k] = on[k] && xa < clo ? t[k][xa] : 0u;
+            vr[k] = on[k] && xr < u1.x ? t[k][xr] : 0u;
+        }
+        for (int x = clo + lane; x < chi; x += 32) {
+            uint32_t v[RB];
+#pragma unroll
+            for (int k = 0; k < RB; ++k) v[k] = on[k] ? t[k][x] : 0u;
+#pragma unroll
+            for (int k = 0; k < RB; ++k) {
+                a1 += v[k];
+                a2 += v[k] * v[k];
             }
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
-            b += __shfl_xor_sync(0xFFFFFFFFu, b, o);
-        }
-        if (lane == 0) {
-            s1[si] = a;
-            s2[si] = b;
+        for (int k = 0; k < RB; ++k) {
+            l1 += va[k];
+            l2 += va[k] * va[k];
+            h1 += vr[k];
+            h2 += vr[k] * vr[k];
         }
     }
+    // the rows outside it
+    const int before = max(min(ylo, u1.y) - u0.y, 0), start = max(yhi, u0.y + before);
+    for (int i = warp; i < before + (u1.y - start); i += WARPS) {
+        const int y = i < before ? u0.y + i : start + (i - before);
+        const uint16_t *t = plane + (size_t)y * X;
+        const uint32_t va = xa < clo ? t[xa] : 0u, vr = xr < u1.x ? t[xr] : 0u;
+        unsigned long long s1 = 0, s2 = 0;
+        for (int x = clo + lane; x < chi; x += 32) {
+            const uint32_t v = t[x];
+            s1 += v;
+            s2 += v * v;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s1 += __shfl_xor_sync(0xFFFFFFFFu, s1, o);
+            s2 += __shfl_xor_sync(0xFFFFFFFFu, s2, o);
+        }
+        for (int sy = 0; sy < SY; ++sy) {
+            const Range w = shared_range(d0.y + sy - r.y, Y, side);
+            if (y < w.lo || y >= w.hi) continue;
+            if (lane == 0) {
+                atomicAdd(&xc[0][sy], s1);
+                atomicAdd(&xc[1][sy], s2);
+            }
+            if (xa < clo) {
+                atomicAdd(&col[0][sy][lane], (unsigned long long)va);
+                atomicAdd(&col[1][sy][lane], (unsigned long long)(va * va));
+            }
+            if (xr < u1.x) {
+                atomicAdd(&col[0][sy][32 + lane], (unsigned long long)vr);
+                atomicAdd(&col[1][sy][32 + lane], (unsigned long long)(vr * vr));
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        a1 += __shfl_xor_sync(0xFFFFFFFFu, a1, o);
+        a2 += __shfl_xor_sync(0xFFFFFFFFu, a2, o);
+    }
+    if (lane == 0) {
+        atomicAdd(&xc[0][SY], a1);
+        atomicAdd(&xc[1][SY], a2);
+    }
+    atomicAdd(&col[0][SY][lane], l1);
+    atomicAdd(&col[1][SY][lane], l2);
+    atomicAdd(&col[0][SY][32 + lane], h1);
+    atomicAdd(&col[1][SY][32 + lane], h2);
+    __syncthreads();
+    const size_t o = P.planes[side] + (size_t)blockIdx.x * SY * SX;
+    for (int i = threadIdx.x; i < SY * SX; i += RP_THREADS) {
+        const int sy = i / SX;
+        const Range wx = shared_range(d0.x + i % SX - r.x, X, side), wy = shared_range(d0.y + sy - r.y, Y, side);
+        unsigned long long s[2] = {0ull, 0ull};
+        if (wx.lo < wx.hi && wy.lo < wy.hi) {
+            for (int k = 0; k < 2; ++k) {
+                s[k] = xc[k][sy] + xc[k][SY];
+                for (int x = wx.lo; x < min(clo, wx.hi); ++x) s[k] += col[k][sy][x - u0.x] + col[k][SY][x - u0.x];
+                for (int x = chi; x < wx.hi; ++x) s[k] += col[k][sy][32 + x - chi] + col[k][SY][32 + x - chi];
+            }
+        }
+        p1[o + i] = s[0];
+        p2[o + i] = s[1];
+    }
+}
+
+// Per shift: the sums of v and v^2 over a side's shared box, one thread per
+// shift adding its planes; block (shifts, 2 pair + side).
+__global__ void k_reg_box(const RegPair *__restrict__ pairs, const unsigned long long *__restrict__ p1,
+                          const unsigned long long *__restrict__ p2, int X, int Y, int Z, int3 r,
+                          unsigned long long *__restrict__ sums, size_t per) {
+    const RegPair &P = pairs[blockIdx.y >> 1];
+    const int side = blockIdx.y & 1;
+    const int3 u0 = P.u0[side], u1 = P.u1[side], d0 = P.d0;
+    const int SX = 2 * r.x + 1, SY = 2 * r.y + 1, S = SX * SY * (2 * r.z + 1);
+    const int si = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (si >= S) return;
+    const Range zr = shared_range(d0.z + si / (SX * SY) - r.z, Z, side);
+    unsigned long long a = 0, b = 0;
+    if (u1.x > u0.x && u1.y > u0.y)
+        for (int z = zr.lo; z < zr.hi; ++z) {
+            const size_t i = P.planes[side] + (size_t)(z - u0.z) * SY * SX + si % (SX * SY);
+            a += p1[i];
+            b += p2[i];
+        }
+    unsigned long long *o = sums + per * (blockIdx.y >> 1) + (size_t)(1 + 2 * side) * S;
+    o[si] = a;
+    o[S + si] = b;
 }
 
 int fail(cudaError_t e) {
@@ -280,55 +408,25 @@ int fail(cudaError_t e) {
         if (e__ != cudaSuccess) return fail(e__); \
     } while (0)
 
-// Device buffers of one registration call, freed on every return path.
-// Device scratch of one call, from the stream-ordered pool on stream s, and
-// REG_STREAMS worker streams that take the pairs in turn.
-constexpr int REG_STREAMS = 4;
-
+// Device scratch of one call, from the stream-ordered pool on its stream s,
+// freed on every return path.
 struct Scratch {
     std::vector<void *> ptrs;
     cudaStream_t s = nullptr;
-    cudaStream_t w[REG_STREAMS] = {};
-    cudaEvent_t ev[REG_STREAMS + 1] = {};
     ~Scratch() {
-        if (s && w[REG_STREAMS - 1] && ev[REG_STREAMS - 1]) join();  // frees wait for the worker streams too
         for (void *p : ptrs) cudaFreeAsync(p, s);
-        if (s) cudaStreamSynchronize(s);
-        for (int k = 0; k < REG_STREAMS; ++k)
-            if (w[k]) cudaStreamDestroy(w[k]);
-        for (int k = 0; k <= REG_STREAMS; ++k)
-            if (ev[k]) cudaEventDestroy(ev[k]);
-        if (s) cudaStreamDestroy(s);
+        if (s) {
+            cudaStreamSynchronize(s);
+            cudaStreamDestroy(s);
+        }
     }
-    cudaError_t init() {
-        cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
-        for (int k = 0; k < REG_STREAMS && e == cudaSuccess; ++k)
-            e = cudaStreamCreateWithFlags(&w[k], cudaStreamNonBlocking);
-        for (int k = 0; k <= REG_STREAMS && e == cudaSuccess; ++k)
-            e = cudaEventCreateWithFlags(&ev[k], cudaEventDisableTiming);
-        return e;
-    }
+    cudaError_t init() { return cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking); }
     template <class T>
     cudaError_t alloc(T **p, size_t n) {
         void *q = nullptr;
         const cudaError_t e = cudaMallocAsync(&q, n ? n * sizeof(T) : 1, s);
         if (e == cudaSuccess) ptrs.push_back(q);
         *p = static_cast<T *>(q);
-        return e;
-    }
-    // the worker streams wait for everything queued on s so far
-    cudaError_t fork() {
-        cudaError_t e = cudaEventRecord(ev[REG_STREAMS], s);
-        for (int k = 0; k < REG_STREAMS && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(w[k], ev[REG_STREAMS], 0);
-        return e;
-    }
-    // s waits for everything queued on the worker streams so far
-    cudaError_t join() {
-        cudaError_t e = cudaSuccess;
-        for (int k = 0; k < REG_STREAMS && e == cudaSuccess; ++k) {
-            e = cudaEventRecord(ev[k], w[k]);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev[k], 0);
-        }
         return e;
     }
 };
@@ -345,43 +443,6 @@ void side_region(const int *d0, const int *r, const int *D, int side, int3 &u0, 
     }
     u0 = make_int3(lo[0], lo[1], lo[2]);
     u1 = make_int3(hi[0], hi[1], hi[2]);
-}
-
-// Entries of the prefix buffers one side of a pair needs.
-void side_sizes(const int *D, const int *d0, const int *r, int side, size_t &np, size_t &nq) {
-    int3 u0, u1;
-    side_region(d0, r, D, side, u0, u1);
-    const size_t UX = (size_t)(u1.x - u0.x), UY = (size_t)(u1.y - u0.y), UZ = (size_t)(u1.z - u0.z);
-    np = (size_t)(2 * r[0] + 1) * UY * UZ * (UX > 0 ? 1 : 0);
-    nq = (size_t)(2 * r[0] + 1) * UZ * (UY + 1);
-}
-
-// Buffers (p1, p2: x-range sums per row; q1, q2: prefixes along y), sized
-// for the largest side.
-struct Prefix {
-    unsigned long long *p1, *p2, *q1, *q2;
-};
-
-// Sa, Saa (side 0) or Sb, Sbb (side 1) of every shift.
-int side_sums(cudaStream_t st, const Prefix &pf, const uint16_t *T, const int *D, const int *d0, const int *r,
-              int side, unsigned long long *s1, unsigned long long *s2) {
-    int3 u0, u1;
-    side_region(d0, r, D, side, u0, u1);
-    const int UX = u1.x - u0.x, UY = u1.y - u0.y, UZ = u1.z - u0.z;
-    const int SX = 2 * r[0] + 1, S = SX * (2 * r[1] + 1) * (2 * r[2] + 1);
-    if (UX <= 0 || UY <= 0 || UZ <= 0) {
-        RK(cudaMemsetAsync(s1, 0, S * sizeof(unsigned long long), st));
-        RK(cudaMemsetAsync(s2, 0, S * sizeof(unsigned long long), st));
-        return SEG_OK;
-    }
-    unsigned long long *p1 = pf.p1, *p2 = pf.p2, *q1 = pf.q1, *q2 = pf.q2;
-    const int rows = UY * UZ;
-    k_reg_rows<<<(rows + 7) / 8, 256, 0, st>>>(T, D[0], D[1], u0, u1, d0[0], r[0], side, p1, p2);
-    k_reg_q<<<SX * UZ, RQ_THREADS, 0, st>>>(p1, p2, u0, u1, q1, q2);
-    k_reg_box<<<(S + 7) / 8, 256, 0, st>>>(q1, q2, D[0], D[1], D[2], u0, u1, make_int3(d0[0], d0[1], d0[2]),
-                                             make_int3(r[0], r[1], r[2]), side, s1, s2);
-    RK(cudaGetLastError());
-    return SEG_OK;
 }
 
 uint32_t uf_root(std::vector<uint32_t> &p, uint32_t i) {
@@ -456,64 +517,64 @@ extern "C" int seg_register_montage(int device, const uint16_t *const *tiles, in
     }
     const int SX = 2 * r[0] + 1, SY = 2 * r[1] + 1, S = SX * SY * (2 * r[2] + 1);
     // Pairs go in groups of up to REG_GROUP: every pair of a group gets its
-    // own slice of sums (Sab, Sa, Saa, Sb, Sbb of every shift), the group's
-    // kernels are queued back to back, and one copy and one synchronisation
-    // bring its sums to the host.
+    // own slice of sums (Sab, Sa, Saa, Sb, Sbb of every shift), each kernel
+    // takes the whole group in one launch, and one copy and one
+    // synchronisation bring its sums to the host.
     constexpr size_t REG_GROUP = 64;
     const size_t per = 5 * (size_t)S;
     const size_t gmax = std::max<size_t>(1, std::min(E.size(), REG_GROUP));
-    unsigned long long *dsum;
-    RK(sc.alloc(&dsum, per * gmax));
-    std::vector<unsigned long long> hs(per * gmax);
-    size_t np = 1, nq = 1;
-    for (const seg_montage_edge &e : E) {
+    unsigned long long *dsum, *dp1, *dp2;
+    RegPair *dpair;
+    std::vector<RegPair> pairs(E.size());
+    size_t npl = 1;  // plane sums of the largest group
+    for (size_t ei = 0, used = 0; ei < E.size(); ++ei) {
+        const seg_montage_edge &e = E[ei];
+        RegPair &P = pairs[ei];
+        if (ei % REG_GROUP == 0) used = 0;
         const int d0[3] = {stage[e.b].x - stage[e.a].x, stage[e.b].y - stage[e.a].y, stage[e.b].z - stage[e.a].z};
+        P.tile[0] = dt[e.a];
+        P.tile[1] = dt[e.b];
+        P.d0 = make_int3(d0[0], d0[1], d0[2]);
         for (int side = 0; side < 2; ++side) {
-            size_t a, b;
-            side_sizes(D, d0, r, side, a, b);
-            np = std::max(np, a);
-            nq = std::max(nq, b);
+            side_region(d0, r, D, side, P.u0[side], P.u1[side]);
+            P.planes[side] = used;
+            used += (size_t)SX * SY * (size_t)(P.u1[side].z - P.u0[side].z);
         }
+        npl = std::max(npl, used);
     }
-    Prefix pf[REG_STREAMS];
-    for (int k = 0; k < REG_STREAMS; ++k) {
-        RK(sc.alloc(&pf[k].p1, np));
-        RK(sc.alloc(&pf[k].p2, np));
-        RK(sc.alloc(&pf[k].q1, nq));
-        RK(sc.alloc(&pf[k].q2, nq));
-    }
+    RK(sc.alloc(&dsum, per * gmax));
+    RK(sc.alloc(&dp1, npl));
+    RK(sc.alloc(&dp2, npl));
+    RK(sc.alloc(&dpair, gmax));
+    std::vector<unsigned long long> hs(per * gmax);
     const size_t smem = reg_corr_smem(r[0], r[1], r[2]);
     const RegCorrFn corr = reg_corr_fn(r[0], std::make_integer_sequence<int, SEG_REG_MAX_RXY + 1>{});
     if (!corr) return SEG_EINVAL;
     RK(cudaFuncSetAttribute(corr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int3 r3 = make_int3(r[0], r[1], r[2]);
     for (size_t g0 = 0; g0 < E.size(); g0 += REG_GROUP) {
         const size_t g1 = std::min(E.size(), g0 + REG_GROUP);
-        RK(sc.fork());
+        const unsigned ng = (unsigned)(g1 - g0);
+        // a pair's blocks: sub-boxes of side 0, planes of either side
+        size_t nb = 0;
+        int nz = 0;
         for (size_t ei = g0; ei < g1; ++ei) {
-            const seg_montage_edge &e = E[ei];
-            unsigned long long *ds = dsum + per * (ei - g0);
-            const int k = (int)(ei % REG_STREAMS);
-            const cudaStream_t st = sc.w[k];
-            const int d0[3] = {stage[e.b].x - stage[e.a].x, stage[e.b].y - stage[e.a].y,
-                               stage[e.b].z - stage[e.a].z};
-            RK(cudaMemsetAsync(ds, 0, S * sizeof(unsigned long long), st));
-            int3 u0, u1;
-            side_region(d0, r, D, 0, u0, u1);
-            if (u1.x > u0.x && u1.y > u0.y && u1.z > u0.z) {
-                const int nb = ((u1.x - u0.x + RC_TX - 1) / RC_TX) * ((u1.y - u0.y + RC_TY - 1) / RC_TY) *
-                               ((u1.z - u0.z + RC_TZ - 1) / RC_TZ);
-                corr<<<nb, RC_THREADS, smem, st>>>(dt[e.a], dt[e.b], D[0], D[1], D[2], u0, u1,
-                                                   make_int3(d0[0], d0[1], d0[2]), r[1], r[2], ds);
-                RK(cudaGetLastError());
-            }
-            int rc = side_sums(st, pf[k], dt[e.a], D, d0, r, 0, ds + S, ds + 2 * (size_t)S);
-            if (rc != SEG_OK) return rc;
-            rc = side_sums(st, pf[k], dt[e.b], D, d0, r, 1, ds + 3 * (size_t)S, ds + 4 * (size_t)S);
-            if (rc != SEG_OK) return rc;
+            const int3 u0 = pairs[ei].u0[0], u1 = pairs[ei].u1[0];
+            nb = std::max(nb, (size_t)((u1.x - u0.x + RC_TX - 1) / RC_TX) * ((u1.y - u0.y + RC_TY - 1) / RC_TY) *
+                                  ((u1.z - u0.z + RC_TZ - 1) / RC_TZ));
+            for (int side = 0; side < 2; ++side) nz = std::max(nz, pairs[ei].u1[side].z - pairs[ei].u0[side].z);
         }
-        RK(sc.join());
-        RK(cudaMemcpyAsync(hs.data(), dsum, per * (g1 - g0) * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                           sc.s));
+        RK(cudaMemcpyAsync(dpair, pairs.data() + g0, ng * sizeof(RegPair), cudaMemcpyHostToDevice, sc.s));
+        RK(cudaMemsetAsync(dsum, 0, per * ng * sizeof(unsigned long long), sc.s));
+        if (nz > 0) {
+            k_reg_plane<<<dim3((unsigned)nz, 2 * ng), RP_THREADS, 0, sc.s>>>(dpair, D[0], D[1], r3, dp1, dp2);
+            k_reg_box<<<dim3((unsigned)((S + 63) / 64), 2 * ng), 64, 0, sc.s>>>(dpair, dp1, dp2, D[0], D[1], D[2], r3,
+                                                                               dsum, per);
+        }
+        if (nb > 0)
+            corr<<<dim3((unsigned)nb, ng), RC_THREADS, smem, sc.s>>>(dpair, D[0], D[1], D[2], r[1], r[2], dsum, per);
+        RK(cudaGetLastError());
+        RK(cudaMemcpyAsync(hs.data(), dsum, per * ng * sizeof(unsigned long long), cudaMemcpyDeviceToHost, sc.s));
         RK(cudaStreamSynchronize(sc.s));
         for (size_t ei = g0; ei < g1; ++ei) {
             seg_montage_edge &e = E[ei];
