@@ -14,7 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libseg.so")
-SOURCES = ["seg_kernels.cu", "seg_runtime.cu", "seg_montage.cu"]
+SOURCES = ["seg_kernels.cu", "seg_box.cu", "seg_runtime.cu", "seg_montage.cu"]
 HEADERS = [os.path.join(CSRC, "seg_internal.h"), os.path.join(INCLUDE, "seg.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -106,7 +106,7 @@ struct VolDev {
     uint16_t *dn_out;         // denoised image (the smoothing's input)
     uint32_t dn_r;            // box radius, 0 = no denoise
     uint32_t dn_mul;          // ceil(2^32 / (2 dn_r + 1)): division by the box width
-    uint32_t dn_n[3];         // box-pass items per axis (lines x chunks)
+    uint32_t dn_n[3];         // box-pass items per axis (groups of lines x chunks)
     uint32_t dn_base0, dn_base1, dn_base2;  // first flat box item per axis
     uint32_t dn_tiles;        // median tiles
     uint32_t dn_tbase;        // first flat median tile
@@ -198,11 +198,11 @@ struct LaunchPlan {
     int grid_ul;         // k_union_local
     int grid_task;       // k_union, k_flatten
     int grid_lab;        // k_label_features
-    int grid_box;        // k_box_pass
+    int grid_box;        // k_box_x, k_box_lines
     int grid_med;        // k_median27
     bool rows;           // some volume of the batch takes k_smooth_rows
     bool tiles;          // some volume of the batch takes k_smooth_hist
-    bool denoise;        // some volume of the batch runs the denoise front end
+    uint32_t denoise;    // denoise front end: bit k set for volumes of radius class k (1..4, 5..8, 9..16)
     bool closing;        // some volume of the batch closes its foreground
     bool distance;       // some volume of the batch has a distance map
     int grid_dist;       // k_dist_x, k_dist_line
@@ -225,11 +225,17 @@ cudaError_t launch_pipeline(const BatchHdr *d_hdr, const LaunchPlan &plan, cudaS
 cudaError_t launch_tile_probe(const BatchHdr *d_hdr, const LaunchPlan &plan, cudaStream_t stream);
 
 // Denoise front end of the volumes with dn_r > 0 (none: the kernels exit).
-constexpr int DN_CHUNK = 128;    // box-pass positions per tile along a line
+constexpr int DN_CHUNK = 256;    // box-pass positions per chunk of a line along y or z ...
+constexpr int DN_CHUNK_X = 128;  // ... and along x
 constexpr int MED_TILE_X = 64, MED_TILE_Y = 8, MED_TILE_Z = 8;  // k_median27 tile (voxels)
 constexpr int DN_MAX_R = 16;
 constexpr int CL_MAX_R = 8;      // closing ball radius limit
 cudaError_t launch_denoise(const BatchHdr *d_hdr, const LaunchPlan &plan, cudaStream_t stream);
+// Box passes (seg_box.cu): items of one axis for `lines` lines of n positions,
+// kernel attributes, and the launches.
+uint32_t box_lines_items(uint64_t lines, uint32_t n, uint32_t chunk);
+cudaError_t configure_box();
+void launch_box_passes(const BatchHdr *d, const LaunchPlan &plan, cudaStream_t s);
 
 // Cell-to-vessel distance: out[k - 1] = min of map over the voxels labelled k.
 cudaError_t launch_cell_distance(const uint32_t *labels, const uint32_t *map, uint64_t n, uint32_t *out, uint64_t k,

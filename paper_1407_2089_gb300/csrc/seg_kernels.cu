@@ -2500,201 +2500,7 @@ __global__ void k_gather_stat(const BatchHdr *__restrict__ h, uint32_t *out) {
 // Eq. 1): background B by box passes, D = max(L - B, 0), 3x3x3 median of D
 // ----------------------------------------------------------------------------
 
-// (n + r) / w for n + r < 2^24 and w = 2r + 1 <= 65, as a multiply-high by
-// mul = ceil(2^32 / w) (division by an invariant integer, Granlund and
-// Montgomery 1994): the product's error n * (mul * w - 2^32) / (w 2^32) stays
-// below 2^-8 < 1/w, so the floor is exact.
-__device__ __forceinline__ uint32_t box_div(uint32_t n, uint32_t mul) { return __umulhi(n, mul); }
-
-// The three rounded box passes of radius r along AXIS, for every tile of 64
-// lines x DN_CHUNK positions of the volumes with the denoise front end.  A
-// block loads its tile with a halo of 3r positions on each side (clamped to
-// the line) into shared memory, runs the three passes there -- pass k over
-// the positions the next one needs, each reading its input at positions
-// clamped to the line, which is the replicate edge of every pass -- and
-// writes the chunk.  Axis x reads dn_src and writes dn_a, y reads dn_a and
-// writes dn_b, z reads dn_b and writes the background into dn_a.  Shared
-// layout [position][lane], lanes padded to 66 so that both the lane-major
-// passes and the position-major copies of axis x avoid bank conflicts.
-constexpr int BOX_LANES = 64, BOX_PITCH = BOX_LANES + 2;
-constexpr int BOX_POS = DN_CHUNK + 6 * DN_MAX_R;
-constexpr size_t BOX_SMEM = 2ull * BOX_POS * BOX_PITCH * sizeof(uint16_t);
-
-template <int AXIS>
-__global__ void __launch_bounds__(256) k_box3(const BatchHdr *__restrict__ h) {
-    __shared__ VolIndex<AXIS == 0 ? &VolDev::dn_base0 : (AXIS == 1 ? &VolDev::dn_base1 : &VolDev::dn_base2)> VI;
-    extern __shared__ __align__(16) uint16_t bsm[];
-    uint16_t *bufA = bsm, *bufB = bsm + BOX_POS * BOX_PITCH;
-    VI.load(h);
-    const int t = threadIdx.x;
-    for (uint32_t it = blockIdx.x; it < h->dn_items[AXIS]; it += gridDim.x) {
-        const VolDev &V = h->vol[VI.find(h, it)];
-        const uint32_t li = it - (AXIS == 0 ? V.dn_base0 : (AXIS == 1 ? V.dn_base1 : V.dn_base2));
-        const int X = (int)V.X, Y = (int)V.Y, Z = (int)V.Z;
-        const int n = AXIS == 0 ? X : (AXIS == 1 ? Y : Z);
-        const int nchunk = (n + DN_CHUNK - 1) / DN_CHUNK;
-        const int group = (int)(li / (uint32_t)nchunk), chunk = (int)(li % (uint32_t)nchunk);
-        const int r = (int)V.dn_r;
-        const uint32_t mul = V.dn_mul;
-        const int c0 = chunk * DN_CHUNK, c1 = min(c0 + DN_CHUNK, n), base = c0 - 3 * r;
-        const int lo = max(base, 0), hi = min(c1 + 3 * r, n);  // loaded positions
-        // lane l of this group: its line's first element and the step along it
-        const int nxg = (X + BOX_LANES - 1) / BOX_LANES;
-        int nl;            // lanes of this group that exist
-        size_t gstart;     // element of lane 0 at position 0
-        size_t lstride, pstride;
-        if (AXIS == 0) {
-            const int rows = Y * Z;
-            nl = min(BOX_LANES, rows - group * BOX_LANES);
-            gstart = (size_t)group * BOX_LANES * X;
-            lstride = (size_t)X;
-            pstride = 1;
-        } else {
-            const int gx = group % nxg, other = group / nxg;
-            nl = min(BOX_LANES, X - gx * BOX_LANES);
-            lstride = 1;
-            if (AXIS == 1) {
-                gstart = (size_t)gx * BOX_LANES + (size_t)X * Y * other;
-                pstride = (size_t)X;
-            } else {
-                gstart = (size_t)gx * BOX_LANES + (size_t)X * other;
-                pstride = (size_t)X * Y;
-            }
-        }
-        const uint16_t *src = AXIS == 0 ? V.dn_src : (AXIS == 1 ? V.dn_a : V.dn_b);
-        uint16_t *dst = AXIS == 1 ? V.dn_b : V.dn_a;
-        const int np = hi - lo;
-        __syncthreads();  // the previous tile is done with the buffers
-        // load: consecutive threads on consecutive elements in memory, eight
-        // independent loads in flight per thread before the shared stores
-        constexpr int NB = 8;
-        if (AXIS == 0) {
-            // one warp per line (a row segment), lanes along it
-            const int lane = t & 31, warp = t >> 5, nw = blockDim.x >> 5;
-            for (int l = warp; l < nl; l += nw) {
-                const uint16_t *row = src + gstart + (size_t)l * lstride;
-                for (int q0 = lo + lane; q0 < hi; q0 += 32 * NB) {
-                    uint16_t v[NB];
-#pragma unroll
-                    for (int j = 0; j < NB; ++j)
-                        if (q0 + 32 * j < hi) v[j] = row[q0 + 32 * j];
-#pragma unroll
-                    for (int j = 0; j < NB; ++j)
-                        if (q0 + 32 * j < hi) bufA[(q0 + 32 * j - base) * BOX_PITCH + l] = v[j];
-                }
-            }
-        } else if ((X & 7) == 0) {
-            // rows of 8-voxel octets (X % 8 == 0, scratch buffers 16-byte
-            // aligned): thread t moves lanes 8 (t % 8) .. + 7 of positions
-            // t / 8 + 32 i as one 16-byte load and four 4-byte shared stores
-            // (pitch 66: the 32 threads of a warp hit 32 different banks)
-            const int oct = t & 7, pr = t >> 3;
-            constexpr int NV = 4;
-            if (8 * oct < nl) {
-                const uint16_t *col = src + gstart + 8 * oct;
-                for (int q0 = lo + pr; q0 < hi; q0 += 32 * NV) {
-                    uint4 v[NV];
-#pragma unroll
-                    for (int j = 0; j < NV; ++j)
-                        if (q0 + 32 * j < hi)
-                            v[j] = *reinterpret_cast<const uint4 *>(col + (size_t)(q0 + 32 * j) * pstride);
-#pragma unroll
-                    for (int j = 0; j < NV; ++j)
-                        if (q0 + 32 * j < hi) {
-                            uint32_t *w = reinterpret_cast<uint32_t *>(bufA + (q0 + 32 * j - base) * BOX_PITCH + 8 * oct);
-                            w[0] = v[j].x; w[1] = v[j].y; w[2] = v[j].z; w[3] = v[j].w;
-                        }
-                }
-            }
-        } else {
-            const int total = np * BOX_LANES, nt = blockDim.x;
-            for (int i0 = t; i0 < total; i0 += nt * NB) {
-                uint16_t v[NB];
-#pragma unroll
-                for (int j = 0; j < NB; ++j) {
-                    const int i = i0 + j * nt, l = i % BOX_LANES, q = lo + i / BOX_LANES;
-                    if (i < total && l < nl) v[j] = src[gstart + (size_t)l * lstride + (size_t)q * pstride];
-                }
-#pragma unroll
-                for (int j = 0; j < NB; ++j) {
-                    const int i = i0 + j * nt, l = i % BOX_LANES, q = lo + i / BOX_LANES;
-                    if (i < total && l < nl) bufA[(q - base) * BOX_PITCH + l] = v[j];
-                }
-            }
-        }
-        __syncthreads();
-        // three passes: A -> B over [c0-2r, c1+2r), B -> A over [c0-r, c1+r), A -> B over [c0, c1)
-        const int l = t % BOX_LANES, seg = t / BOX_LANES;
-        for (int k = 0; k < 3; ++k) {
-            const uint16_t *in = (k == 1) ? bufB : bufA;
-            uint16_t *out = (k == 1) ? bufA : bufB;
-            const int p0 = max(c0 - (2 - k) * r, 0), p1 = min(c1 + (2 - k) * r, n);
-            const int per = (p1 - p0 + 3) / 4;
-            const int q0 = p0 + seg * per, q1 = min(q0 + per, p1);
-            if (l < nl && q0 < q1) {
-                // every read lies in [q0 - r, q1 - 1 + r] clamped to the line,
-                // inside the positions the previous pass (or the load) covered
-                auto at = [&](int q) { return (uint32_t)in[(min(max(q, 0), n - 1) - base) * BOX_PITCH + l]; };
-                // sum holds the window sum plus the rounding term r
-                uint32_t sum = (uint32_t)r;
-                if (q0 - r >= 0 && q0 + r < n) {
-                    const uint16_t *pw = in + (q0 - r - base) * BOX_PITCH + l;
-                    for (int i = 0; i <= 2 * r; ++i) sum += pw[i * BOX_PITCH];
-                } else {
-                    for (int q = q0 - r; q <= q0 + r; ++q) sum += at(q);
-                }
-                out[(q0 - base) * BOX_PITCH + l] = (uint16_t)box_div(sum, mul);
-                // positions q whose window [q - r - 1, q + r] needs no
-                // clamping run through three moving pointers
-                const int qa = min(max(q0 + 1, r + 1), q1), qb = max(min(q1, n - r), qa);
-                int q = q0 + 1;
-                for (; q < qa; ++q) {
-                    sum += at(q + r) - at(q - r - 1);
-                    out[(q - base) * BOX_PITCH + l] = (uint16_t)box_div(sum, mul);
-                }
-                const uint16_t *pin = in + (q + r - base) * BOX_PITCH + l;
-                const uint16_t *pout = in + (q - r - 1 - base) * BOX_PITCH + l;
-                uint16_t *po = out + (q - base) * BOX_PITCH + l;
-#pragma unroll 4
-                for (; q < qb; ++q) {
-                    sum += (uint32_t)*pin - (uint32_t)*pout;
-                    *po = (uint16_t)box_div(sum, mul);
-                    pin += BOX_PITCH;
-                    pout += BOX_PITCH;
-                    po += BOX_PITCH;
-                }
-                for (; q < q1; ++q) {
-                    sum += at(q + r) - at(q - r - 1);
-                    out[(q - base) * BOX_PITCH + l] = (uint16_t)box_div(sum, mul);
-                }
-            }
-            __syncthreads();
-        }
-        // store the chunk from B
-        const int nc = c1 - c0;
-        if (AXIS == 0) {
-            const int lane = t & 31, warp = t >> 5, nw = blockDim.x >> 5;
-            for (int ll = warp; ll < nl; ll += nw) {
-                uint16_t *row = dst + gstart + (size_t)ll * lstride;
-                for (int q = c0 + lane; q < c1; q += 32) row[q] = bufB[(q - base) * BOX_PITCH + ll];
-            }
-        } else if ((X & 7) == 0) {
-            const int oct = t & 7, pr = t >> 3;
-            if (8 * oct < nl) {
-                uint16_t *col = dst + gstart + 8 * oct;
-                for (int q = c0 + pr; q < c1; q += 32) {
-                    const uint32_t *w = reinterpret_cast<const uint32_t *>(bufB + (q - base) * BOX_PITCH + 8 * oct);
-                    *reinterpret_cast<uint4 *>(col + (size_t)q * pstride) = make_uint4(w[0], w[1], w[2], w[3]);
-                }
-            }
-        } else {
-            for (int i = t; i < nc * BOX_LANES; i += blockDim.x) {
-                const int ll = i % BOX_LANES, q = c0 + i / BOX_LANES;
-                if (ll < nl) dst[gstart + (size_t)ll * lstride + (size_t)q * pstride] = bufB[(q - base) * BOX_PITCH + ll];
-            }
-        }
-    }
-}
+// (the box passes are in seg_box.cu)
 
 // D = max(L - B, 0) staged per tile of 64 x 8 x 8 voxels (plus a one-voxel
 // halo, clamped), then the median of each voxel's 27 neighbours from the
@@ -4270,15 +4076,8 @@ cudaError_t configure_kernels(int device, LaunchPlan &plan) {
     if ((e = resident((const void *)k_flatten, ROW_TILE, &g2)) != cudaSuccess) return e;
     plan.grid_task = std::min(g1, g2);
     if ((e = resident((const void *)k_label_features, ROW_TILE, &plan.grid_lab)) != cudaSuccess) return e;
-    for (const void *fn : {(const void *)k_box3<0>, (const void *)k_box3<1>, (const void *)k_box3<2>})
-        if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BOX_SMEM)) != cudaSuccess)
-            return e;
-    {
-        int per_sm = 0;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_box3<1>, 256, BOX_SMEM)) != cudaSuccess)
-            return e;
-        plan.grid_box = plan.sms * (per_sm > 0 ? per_sm : 1);
-    }
+    if ((e = configure_box()) != cudaSuccess) return e;
+    plan.grid_box = 16 * plan.sms;  // every class's resident blocks, at most
     if ((e = resident((const void *)k_median27, MED_TX * MED_TY, &plan.grid_med)) != cudaSuccess) return e;
     if ((e = resident((const void *)k_dist_x, 256, &g1)) != cudaSuccess) return e;
     if ((e = resident((const void *)k_dist_line<2>, 256, &g2)) != cudaSuccess) return e;
@@ -4316,12 +4115,6 @@ cudaError_t launch_tile_probe(const BatchHdr *d, const LaunchPlan &p, cudaStream
         default: k_smooth_hist<64><<<p.grid_hist, Tile<64>::NT, hist_smem_bytes(64), s>>>(d); break;
     }
     return cudaGetLastError();
-}
-
-static void launch_box_passes(const BatchHdr *d, const LaunchPlan &p, cudaStream_t s) {
-    k_box3<0><<<p.grid_box, 256, BOX_SMEM, s>>>(d);
-    k_box3<1><<<p.grid_box, 256, BOX_SMEM, s>>>(d);
-    k_box3<2><<<p.grid_box, 256, BOX_SMEM, s>>>(d);
 }
 
 cudaError_t launch_cell_distance(const uint32_t *labels, const uint32_t *map, uint64_t n, uint32_t *out, uint64_t k,

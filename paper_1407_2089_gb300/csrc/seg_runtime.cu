@@ -182,6 +182,7 @@ struct Batch {
     uint32_t nvol = 0;
     uint64_t voxels = 0;
     uint32_t mrf_iters = 0;  // MRF steps launched (the largest limit in the batch)
+    uint32_t dn_classes = 0; // radius classes of the denoise front end in the batch
     std::atomic<bool> done{false};
     int launch_err = SEG_OK;
     struct seg_ctx *ctx = nullptr;
@@ -409,7 +410,7 @@ void build_header(seg_ctx *ctx, Batch &b) {
     const uint32_t rtile = batch_row_tile(ctx, b), lbk = batch_label_shrink(ctx, b);
     const uint64_t bkv = batch_brick_voxels(ctx, b);
     uint32_t fst = 0, lbs = 0;
-    uint32_t v = 0, tiles = 0, rts = 0, bks = 0, bts = 0, dn[3] = {0, 0, 0}, dnt = 0, cl = 0;
+    uint32_t v = 0, tiles = 0, rts = 0, bks = 0, bts = 0, dn[3] = {0, 0, 0}, dnt = 0, cl = 0, dn_classes = 0;
     uint32_t dtb[DT_NK] = {0, 0, 0, 0, 0, 0};
     uint32_t mrft = 0, mrf_iters = 0;
     uint64_t mrfu = 0;
@@ -435,10 +436,10 @@ void build_header(seg_ctx *ctx, Batch &b) {
                 V.raw = V.dn_out;  // the smoothing reads the denoised image
                 const uint64_t w = 2ull * g.dn_r + 1;
                 V.dn_mul = (uint32_t)(((1ull << 32) + w - 1) / w);
-                // tiles of 64 lines x DN_CHUNK positions per axis
-                V.dn_n[0] = (uint32_t)(cdiv((uint64_t)g.Y * g.Z, 64) * cdiv(g.X, DN_CHUNK));
-                V.dn_n[1] = (uint32_t)(cdiv(g.X, 64) * g.Z * cdiv(g.Y, DN_CHUNK));
-                V.dn_n[2] = (uint32_t)(cdiv(g.X, 64) * g.Y * cdiv(g.Z, DN_CHUNK));
+                V.dn_n[0] = box_lines_items(g.rows, g.X, DN_CHUNK_X);
+                V.dn_n[1] = box_lines_items((uint64_t)g.X * g.Z, g.Y, DN_CHUNK);
+                V.dn_n[2] = box_lines_items((uint64_t)g.X * g.Y, g.Z, DN_CHUNK);
+                dn_classes |= g.dn_r <= 4u ? 1u : (g.dn_r <= 8u ? 2u : 4u);
                 V.dn_tiles = (uint32_t)(cdiv(g.X, MED_TILE_X) * cdiv(g.Y, MED_TILE_Y) * cdiv(g.Z, MED_TILE_Z));
             }
             V.dn_base0 = dn[0];
@@ -605,6 +606,7 @@ void build_header(seg_ctx *ctx, Batch &b) {
     h->dn_items[1] = dn[1];
     h->dn_items[2] = dn[2];
     h->dn_tiles = dnt;
+    b.dn_classes = dn_classes;
     h->cl_items = cl;
     for (int k = 0; k < DT_NK; ++k) h->dt_items[k] = dtb[k];
     h->mrf_tiles = mrft;
@@ -618,7 +620,7 @@ void build_header(seg_ctx *ctx, Batch &b) {
 // A captured graph fixes which optional kernels launch and how many MRF steps.
 uint64_t graph_key(const LaunchPlan &p) {
     return (uint64_t)p.tile_y | (uint64_t)p.rows << 11 | (uint64_t)p.tiles << 12 |
-           (uint64_t)p.denoise << 8 | (uint64_t)p.closing << 9 | (uint64_t)p.distance << 10 |
+           (uint64_t)p.denoise << 40 | (uint64_t)p.closing << 9 | (uint64_t)p.distance << 10 |
            (uint64_t)p.mrf_iters << 16;
 }
 
@@ -700,7 +702,7 @@ int launch_batch(seg_ctx *ctx, Batch &b) {
     }
     ctx->plan.rows = s.h_hdr->fs_tiles > 0;
     ctx->plan.tiles = s.h_hdr->ntiles > 0;
-    ctx->plan.denoise = s.h_hdr->dn_tiles > 0;
+    ctx->plan.denoise = b.dn_classes;
     ctx->plan.closing = s.h_hdr->cl_items > 0;
     ctx->plan.distance = false;
     for (int k = 0; k < DT_NK; ++k) ctx->plan.distance |= s.h_hdr->dt_items[k] > 0;
@@ -961,7 +963,7 @@ int seg_create(const seg_config *cfg, seg_ctx **out) {
     ctx->plan.grid_hist = ctx->sms;  // one resident block per SM (176 KiB histogram)
     ctx->plan.grid_vols = ctx->sms;
     ctx->plan.rows = ctx->plan.tiles = true;
-    ctx->plan.denoise = false;
+    ctx->plan.denoise = 0;
     ctx->plan.closing = false;
     ctx->plan.distance = false;
     ctx->plan.mrf_iters = 0;
