@@ -1780,10 +1780,18 @@ __global__ void __launch_bounds__(ROW_TILE) k_threshold_runs(const BatchHdr *__r
     }
 }
 
+// Run table of every row (its runs' offsets from the row counts and the row
+// tiles below).  One thread per row walks its mask words; rows of more than
+// ROW_RUNS_W words take a warp, a lane per word, ranked by a shuffle scan (a
+// thread per row took 415 us for 5530 x 5530 x 80, a warp 309).
+constexpr uint32_t ROW_RUNS_W = 32;
+
 __global__ void __launch_bounds__(ROW_TILE) k_row_runs(const BatchHdr *__restrict__ h) {
     __shared__ VolIndex<&VolDev::rt_base> VI;
     VI.load(h);
     __shared__ uint32_t sbuf[33];
+    __shared__ uint32_t soff[ROW_TILE + 1];  // wide rows: run offsets of the tile's rows
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (uint32_t rt = blockIdx.x; rt < h->nrowtiles; rt += gridDim.x) {
         const VolDev &V = h->vol[VI.find(h, rt)];
         const uint32_t lt = rt - V.rt_base;
@@ -1801,7 +1809,7 @@ __global__ void __launch_bounds__(ROW_TILE) k_row_runs(const BatchHdr *__restric
             const uint32_t off = base + ex;
             V.rowoff[row] = off;
             if (row == V.rows - 1) V.rowoff[V.rows] = off + cnt;
-            if (cnt && off + cnt <= V.r_cap) {
+            if (V.W <= ROW_RUNS_W && cnt && off + cnt <= V.r_cap) {
                 const uint32_t *m = V.mask + (size_t)row * V.W;
                 uint32_t p = 0, k = off;
                 const uint32_t kend = off + cnt;
@@ -1816,6 +1824,42 @@ __global__ void __launch_bounds__(ROW_TILE) k_row_runs(const BatchHdr *__restric
                     p = e + 1;
                 }
             }
+        }
+        if (V.W > ROW_RUNS_W) {  // the same in every thread
+            if (threadIdx.x < h->row_tile) soff[threadIdx.x] = base + ex;
+            if (threadIdx.x == 0) soff[h->row_tile] = base + tot;
+            __syncthreads();
+            const uint32_t row0 = lt * h->row_tile, nrows = min(h->row_tile, V.rows - row0);
+            for (uint32_t r = warp; r < nrows; r += ROW_TILE / 32) {
+                uint32_t k = soff[r];
+                const uint32_t kend = soff[r + 1];
+                if (k == kend || kend > V.r_cap) continue;
+                const uint32_t *m = V.mask + (size_t)(row0 + r) * V.W;
+                uint32_t carry = 0;
+                for (uint32_t w0 = 0; w0 < V.W && k < kend; w0 += 32) {
+                    const uint32_t w = w0 + lane, word = w < V.W ? m[w] : 0u;
+                    uint32_t left = __shfl_up_sync(FULL, word, 1) >> 31;
+                    if (lane == 0) left = carry;
+                    carry = __shfl_sync(FULL, word, 31) >> 31;
+                    uint32_t starts = word & ~(word << 1 | left);
+                    uint32_t n = __popc(starts), at = n;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const uint32_t b = __shfl_up_sync(FULL, at, o);
+                        if ((int)lane >= o) at += b;
+                    }
+                    const uint32_t all = __shfl_sync(FULL, at, 31);
+                    for (uint32_t q = k + at - n; starts; starts &= starts - 1u, ++q) {
+                        const uint32_t s = 32u * w + __ffs(starts) - 1u;
+                        const uint32_t e = find_bit(m, V.W, V.X, s, false) - 1u;
+                        V.run_x[q] = s | (e << 16);
+                        V.run_par[q] = q;
+                        V.run_aux[q] = 0;
+                    }
+                    k += all;
+                }
+            }
+            __syncthreads();  // soff is reused
         }
     }
 }
@@ -2138,18 +2182,44 @@ __global__ void __launch_bounds__(ROW_TILE) k_union(const BatchHdr *__restrict__
     }
 }
 
-// One thread per run (all volumes of the batch in turn): parent = root, and
-// the run's voxels are added to the root's size, one atomic per warp when all
-// its lanes share a root.
+// One thread per run: parent = root, and the run's voxels are added to the
+// root's size, one atomic per warp when all its lanes share a root.  The runs
+// of all volumes are dealt out as one sequence of warps: the blocks work out
+// where each volume's begin (its run count is only known on the device) from
+// one load and a scan; volume after volume instead, every volume waited for
+// the latency of the one before (48 us for 32 channels of 45 000 runs each,
+// 23 as one sequence).  Batches of more than SMEM_VOLS volumes take
+// SMEM_VOLS of them at a time.
 __global__ void __launch_bounds__(ROW_TILE) k_flatten(const BatchHdr *__restrict__ h) {
-    const uint32_t stride = gridDim.x * blockDim.x;
-    const uint32_t lane = threadIdx.x & 31;
-    for (uint32_t v = 0; v < h->nvol; ++v) {
-        const VolDev &V = h->vol[v];
-        const uint32_t R = V.rowoff[V.rows];
+    __shared__ uint32_t base[SMEM_VOLS + 1];  // first warp of each volume
+    __shared__ uint32_t sbuf[33];
+    static_assert(SMEM_VOLS % ROW_TILE == 0, "whole scan rounds");
+    const uint32_t lane = threadIdx.x & 31, nv = h->nvol;
+    const uint32_t warps = gridDim.x * (ROW_TILE / 32);
+    for (uint32_t v0 = 0; v0 < nv; v0 += SMEM_VOLS) {
+        const uint32_t n = min(SMEM_VOLS, nv - v0);
+        uint32_t total = 0;
+        for (uint32_t k = 0; k < n; k += ROW_TILE) {
+            const uint32_t i = k + threadIdx.x;
+            uint32_t w = 0, t;
+            if (i < n) {
+                const VolDev &V = h->vol[v0 + i];
+                w = (V.rowoff[V.rows] + 31u) / 32u;
+            }
+            const uint32_t ex = block_exscan<ROW_TILE>(w, &t, sbuf);
+            if (i < n) base[i] = total + ex;
+            total += t;
+        }
+        __syncthreads();
         // whole warps stay in the loop so that the shuffles see every lane
-        for (uint32_t j0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); j0 < R; j0 += stride) {
-            const uint32_t j = j0 + lane;
+        for (uint32_t u = blockIdx.x * (ROW_TILE / 32) + (threadIdx.x >> 5); u < total; u += warps) {
+            uint32_t lo = 0, hi = n;  // the last volume that begins at or before u
+            while (hi - lo > 1) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (base[mid] <= u) lo = mid; else hi = mid;
+            }
+            const VolDev &V = h->vol[v0 + lo];
+            const uint32_t R = V.rowoff[V.rows], j = (u - base[lo]) * 32u + lane;
             uint32_t root = 0xFFFFFFFFu, len = 0;
             if (j < R) {
                 root = uf_root(V.run_par, j);
@@ -2167,6 +2237,7 @@ __global__ void __launch_bounds__(ROW_TILE) k_flatten(const BatchHdr *__restrict
                 atomicAdd(V.run_aux + root, len);
             }
         }
+        __syncthreads();  // base is rewritten
     }
 }
 
