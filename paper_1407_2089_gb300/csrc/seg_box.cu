@@ -175,18 +175,15 @@ __global__ void __launch_bounds__(BX_THREADS) k_box_lines(const BatchHdr *__rest
         const VolDev &V = h->vol[box_volume<AXIS>(h, it)];
         if (box_class(V.dn_r) != CLS) continue;
         const uint32_t li = it - box_base<AXIS>(V);
-        const int n = (int)(AXIS == 1 ? V.Y : V.Z), nchunk = (n + DN_CHUNK - 1) / DN_CHUNK;
-        const int per = (n + nchunk - 1) / nchunk;
-        const uint32_t group = li / (uint32_t)nchunk;
-        const int c0 = (int)(li % (uint32_t)nchunk) * per, c1 = min(c0 + per, n);
-        const uint64_t line = (uint64_t)group * BX_THREADS + threadIdx.x;
-        if (line >= (uint64_t)V.X * (AXIS == 1 ? V.Z : V.Y) || c0 >= c1) continue;
-        const size_t plane = (size_t)V.X * V.Y;
-        const size_t o = AXIS == 1 ? line / V.X * plane + line % V.X : (size_t)line;
+        const uint32_t len = AXIS == 1 ? V.Y : V.Z, nchunk = box_chunks(len, DN_CHUNK);
+        const BoxChunk c = box_chunk(len, DN_CHUNK, li % nchunk, V.dn_r);
+        const uint64_t line = (uint64_t)(li / nchunk) * BX_THREADS + threadIdx.x;
+        if (line >= (uint64_t)V.X * (AXIS == 1 ? V.Z : V.Y) || c.c0 >= c.c1) continue;
+        const size_t plane = (size_t)V.X * V.Y, st = AXIS == 1 ? (size_t)V.X : plane;
+        const size_t o = (AXIS == 1 ? line / V.X * plane + line % V.X : (size_t)line) + c.first * st;
         const uint16_t *src = AXIS == 1 ? V.dn_a : V.dn_b;
         uint16_t *dst = AXIS == 1 ? V.dn_b : V.dn_a;
-        box_line_r<CLS>((int)V.dn_r, src + o, dst + o, AXIS == 1 ? (size_t)V.X : plane, n, c0, c1, V.dn_mul,
-                        c0 <= 3 * (int)V.dn_r);
+        box_line_r<CLS>((int)V.dn_r, src + o, dst + o, st, c.n, c.c0, c.c1, V.dn_mul, c.start);
     }
 }
 
@@ -256,7 +253,7 @@ void launch_class(const BatchHdr *d, const LaunchPlan &p, cudaStream_t s) {
 }  // namespace
 
 uint32_t box_lines_items(uint64_t lines, uint32_t n, uint32_t chunk) {
-    return (uint32_t)((lines + BX_THREADS - 1) / BX_THREADS * ((n + chunk - 1) / chunk));
+    return (uint32_t)((lines + BX_THREADS - 1) / BX_THREADS * box_chunks(n, chunk));
 }
 
 cudaError_t configure_box() {

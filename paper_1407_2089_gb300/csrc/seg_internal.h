@@ -231,6 +231,27 @@ constexpr int MED_TILE_X = 64, MED_TILE_Y = 8, MED_TILE_Z = 8;  // k_median27 ti
 constexpr int DN_MAX_R = 16;
 constexpr int CL_MAX_R = 8;      // closing ball radius limit
 cudaError_t launch_denoise(const BatchHdr *d_hdr, const LaunchPlan &plan, cudaStream_t stream);
+// A line's chunk in the box passes: its outputs [c0, c1), in positions from
+// `first` on (the first position read; 3 r before the chunk, or the line's
+// start).  Relative positions keep the kernels' 32-bit arithmetic exact for
+// lines of up to SEG_MAX_YZ positions, whose ends leave no room for a chunk's
+// halo below 2^31.
+struct BoxChunk {
+    uint32_t first;
+    int n;           // positions of the line from `first` on
+    int c0, c1;      // none when c0 >= c1
+    bool start;      // `first` is the line's own start
+};
+__host__ __device__ inline uint32_t box_chunks(uint32_t n, uint32_t chunk) {
+    return n / chunk + (n % chunk != 0u ? 1u : 0u);
+}
+// Chunk k of a line of n positions in box_chunks(n, chunk) equal chunks.
+__host__ __device__ inline BoxChunk box_chunk(uint32_t n, uint32_t chunk, uint32_t k, uint32_t r) {
+    const uint32_t per = box_chunks(n, box_chunks(n, chunk)), at = k * per;
+    if (at >= n) return BoxChunk{0u, 0, 0, 0, false};
+    const uint32_t lead = at < 3u * r ? at : 3u * r, len = n - at < per ? n - at : per;
+    return BoxChunk{at - lead, (int)(n - (at - lead)), (int)lead, (int)(lead + len), at == lead};
+}
 // Box passes (seg_box.cu): items of one axis for `lines` lines of n positions,
 // kernel attributes, and the launches.
 uint32_t box_lines_items(uint64_t lines, uint32_t n, uint32_t chunk);
