@@ -300,10 +300,40 @@ cudaError_t launch_label_runs_write(const uint32_t *labels, uint32_t X, uint32_t
                                     const uint32_t *tiles, const uint32_t *total, uint64_t cap, seg_label_run *out,
                                     seg_label_run *mapped, int sms, cudaStream_t s);
 
-// z-chunk for `columns` tile columns of Z planes on `blocks` blocks that take
-// equal shares of the tiles: the one whose fullest block smooths the fewest
-// planes, the four halo planes of each tile counted.
-uint32_t hist_tile_z(uint64_t columns, uint32_t Z, uint32_t blocks);
+// Tile height and z-chunk of seg_otsu_threshold_noalloc for one volume on
+// `blocks` blocks that take equal shares of the tiles: the pair whose fullest
+// block takes the least time, the four halo planes of each tile counted.  A
+// 64-row plane costs 1.4 times a 32-row one (1.6 and 1.15 us), so 64 rows are
+// better for whole tiles (701 x 512 x 64: 77 us against 95; 141 with 32 rows and
+// 64 planes whatever the volume: 176 tiles are two rounds of 152 blocks, the
+// second nearly empty), and 32 where most of a tile's rows would lie past the
+// volume (4096 x 32 x 256: 160 us for the call, 220 with 64 rows).  Fewer columns
+// than blocks are tried in the most chunks that fit 1 to 64 rounds of the blocks,
+// so that a lone column is cut as often as there are blocks (64 x 64 x 20000:
+// 253 us, 530 in at most 64 chunks, 394 in chunks of 64 planes); others in 1 to
+// 64 chunks.
+struct HistSplit {
+    uint32_t ty, tz;
+};
+inline HistSplit hist_split(uint32_t X, uint32_t Y, uint32_t Z, uint32_t blocks) {
+    HistSplit best{64u, Z};
+    uint64_t cost = UINT64_MAX;
+    for (uint32_t ty = 64u; ty >= 32u; ty /= 2u) {
+        const uint64_t columns = ((uint64_t)X + TILE_X - 1) / TILE_X * (((uint64_t)Y + ty - 1) / ty);
+        for (uint32_t k = 1; k <= 64u; ++k) {
+            const uint64_t most = columns < blocks ? (uint64_t)k * blocks / columns : k;
+            const uint32_t n = most < Z ? (uint32_t)most : Z, tz = (Z - 1) / n + 1;
+            const uint64_t tiles = columns * ((Z - 1) / tz + 1);
+            const uint64_t c = (tiles + blocks - 1) / blocks * (tz + 4ull) * (ty == 64u ? 7u : 5u);
+            if (c < cost) {
+                cost = c;
+                best = HistSplit{ty, tz};
+            }
+            if (n == Z) break;
+        }
+    }
+    return best;
+}
 
 // Histogram-kernel shared memory per block for a tile height.
 size_t hist_smem_bytes(int tile_y);

@@ -4109,20 +4109,6 @@ static size_t dxy_smem(int nb) { return 2ull * 2 * 32 * 32 * (size_t)nb; }
 // k_dist_z: uint32 values and byte positions (rows of four, padded)
 constexpr size_t DZ_SMEM = 5ull * DZ_ELEMS + 512;
 
-uint32_t hist_tile_z(uint64_t columns, uint32_t Z, uint32_t blocks) {
-    uint32_t best = Z;
-    uint64_t cost = UINT64_MAX;
-    for (uint32_t n = 1; n <= Z && n <= 64u; ++n) {
-        const uint32_t tz = (Z + n - 1) / n;
-        const uint64_t tiles = columns * ((Z + tz - 1) / tz), c = (tiles + blocks - 1) / blocks * (tz + 4ull);
-        if (c < cost) {
-            cost = c;
-            best = tz;
-        }
-    }
-    return best;
-}
-
 size_t hist_smem_bytes(int tile_y) {
     return tile_y == 16 ? Tile<16>::HIST_SMEM : (tile_y == 32 ? Tile<32>::HIST_SMEM : Tile<64>::HIST_SMEM);
 }
@@ -4345,10 +4331,6 @@ constexpr int NOALLOC_WORDS = HIST_BINS + ST_WORDS;  // 262,208 bytes per device
 // Every GPU that loads the library holds it until the process exits.
 static __device__ __align__(256) uint32_t g_noalloc_scratch[NOALLOC_WORDS];
 
-// 64 rows: 76 us for 701 x 512 x 64, where 32 rows take 95 and 16 rows 150
-// (141 with 32 rows and z-chunks of 64 planes whatever the volume: 176 tiles
-// are two rounds on 152 blocks, the second nearly empty)
-constexpr int NOALLOC_TY = 64;
 constexpr int NOALLOC_MAX_DEVICES = 64;
 
 // Device address of g_noalloc_scratch per device (host code must not use the
@@ -4376,12 +4358,11 @@ __global__ void __launch_bounds__(8 * TY, 1) k_smooth_hist_noalloc(const __grid_
     const uint32_t tb = (uint32_t)(((uint64_t)nt * blockIdx.x) / G);
     const uint32_t te = (uint32_t)(((uint64_t)nt * (blockIdx.x + 1)) / G);
     if (tb >= te) return;
-    const int tz = (int)h->tile_z;
     for (uint32_t t = tb; t < te; ++t) {
         const uint32_t ix = t % V.ntx, rest = t / V.ntx;
         const uint32_t iy = rest % V.nty, iz = rest / V.nty;
-        const int z0 = (int)iz * tz;
-        const int z1 = min(z0 + tz, (int)V.Z);
+        const int z0 = (int)(iz * h->tile_z);
+        const int z1 = (int)min(iz * h->tile_z + h->tile_z, V.Z);  // (up to Z + chunks: unsigned)
         HistEmit<false> e{sh, V.hist, nullptr, V.X, V.Y, 0u, 0u, 0u, nullptr, 0, false};
         smooth_tile<TY>(V.raw, V.X, V.Y, V.Z, (int)ix * TILE_X, (int)iy * TY, z0, z1, spx, R, e);
     }
@@ -4397,9 +4378,11 @@ int noalloc_setup(int dev, uint32_t **ptr, int *sms) {
         void *p = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
         if (e != cudaSuccess) { cudaGetLastError(); return SEG_ECUDA; }
-        e = cudaFuncSetAttribute(k_smooth_hist_noalloc<NOALLOC_TY>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)hist_smem_bytes(NOALLOC_TY));
+        e = cudaFuncSetAttribute(k_smooth_hist_noalloc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)hist_smem_bytes(64));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_smooth_hist_noalloc<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)hist_smem_bytes(32));
         if (e != cudaSuccess) { cudaGetLastError(); return SEG_ECUDA; }
         e = cudaFuncSetAttribute(k_otsu_one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OTSU_SMEM);
         if (e != cudaSuccess) { cudaGetLastError(); return SEG_ECUDA; }
@@ -4443,17 +4426,20 @@ extern "C" int seg_otsu_threshold_noalloc(const uint16_t *d_voxels, seg_dims dim
     V.stat = scratch + HIST_BINS;
     V.X = dims.x; V.Y = dims.y; V.Z = dims.z;
     V.ntx = (uint32_t)(((uint64_t)dims.x + TILE_X - 1) / TILE_X);
-    V.nty = (uint32_t)(((uint64_t)dims.y + NOALLOC_TY - 1) / NOALLOC_TY);
-    const uint32_t tz = hist_tile_z((uint64_t)V.ntx * V.nty, dims.z, (uint32_t)sms);
-    V.ntz = (dims.z + tz - 1) / tz;
+    const HistSplit sp = hist_split(dims.x, dims.y, dims.z, (uint32_t)sms);
+    V.nty = (uint32_t)(((uint64_t)dims.y + sp.ty - 1) / sp.ty);
+    V.ntz = (dims.z - 1) / sp.tz + 1;
     hdr.nvol = 1;
     hdr.ntiles = V.ntx * V.nty * V.ntz;
-    hdr.tile_z = tz;
-    hdr.tile_y = NOALLOC_TY;
+    hdr.tile_z = sp.tz;
+    hdr.tile_y = sp.ty;
     // the array keeps the previous call's contents: clear bins and counters
     cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(uint32_t) * NOALLOC_WORDS, s);
     if (e == cudaSuccess) {
-        k_smooth_hist_noalloc<NOALLOC_TY><<<sms, Tile<NOALLOC_TY>::NT, hist_smem_bytes(NOALLOC_TY), s>>>(hdr);
+        if (sp.ty == 64u)
+            k_smooth_hist_noalloc<64><<<sms, Tile<64>::NT, hist_smem_bytes(64), s>>>(hdr);
+        else
+            k_smooth_hist_noalloc<32><<<sms, Tile<32>::NT, hist_smem_bytes(32), s>>>(hdr);
         k_otsu_one<<<1, OTSU_NT, OTSU_SMEM, s>>>(V.hist, V.stat, n);
         e = cudaGetLastError();
     }
