@@ -53,13 +53,11 @@ __host__ __device__ inline Range shared_range(int d, int D, int side) {
 }
 
 // One overlapping pair on the device: tile b's origin in tile a's frame, the
-// search region of each side (0: a, 1: b) in that tile's frame, and where the
-// plane sums of each side start.
+// search region of each side (0: a, 1: b) in that tile's frame.
 struct RegPair {
     const uint16_t *tile[2];
     int3 d0;
     int3 u0[2], u1[2];
-    size_t planes[2];
 };
 
 // Sab for every shift: block (x, y) = sub-box x (RC_TX x RC_TY x RC_TZ) of the
@@ -73,10 +71,13 @@ struct RegPair {
 // moved to 64-bit sums; only where one row could overflow are the sums 64-bit
 // throughout (three instructions per product instead of one).  Bound by
 // instruction issue (one multiply-add per product, a third more for staging
-// and unpacking): 1.93 ms for the 20.5 G products of 3 x 3 tiles of 1024 x 1024
+// and unpacking): 1.83 ms for the 20.5 G products of 3 x 3 tiles of 1024 x 1024
 // x 64 with a tenth of overlap and radius 4, 4, 1, where 64-bit sums over 8 x 8
-// rows took 3.2 ms; 8 x 16 rows take 2.1 ms.  The threads' sums meet in shared memory and go out with one atomic
-// per (block, shift).
+// rows took 3.2 ms; 8 x 16 rows take 2.1 ms.  Wider windows stage more per block
+// (75 KB at radius 6, 6, 2, 211 KB at 12, 12, 6) and gain less: whole calls of 2 x
+// 2 tiles of 1024 x 1024 x 64 at 6, 6, 2 take 2.81 ms against 3.48, of two tiles of
+// 1024 x 1024 x 32 at 12, 12, 6 3.31 against 3.85.  The threads' sums meet in
+// shared memory and go out with one atomic per (block, shift).
 template <int RX>
 __global__ void __launch_bounds__(RC_THREADS) k_reg_corr(const RegPair *__restrict__ pairs, int X, int Y, int Z, int ry,
                                                          int rz, unsigned long long *__restrict__ sums, size_t per) {
@@ -88,7 +89,7 @@ __global__ void __launch_bounds__(RC_THREADS) k_reg_corr(const RegPair *__restri
     const uint16_t *__restrict__ A = P.tile[0], *__restrict__ B = P.tile[1];
     const int3 u0 = P.u0[0], u1 = P.u1[0], d0 = P.d0;
     unsigned long long *sab = sums + per * blockIdx.y;
-    const int BY = RC_TY + 2 * ry, BZ = RC_TZ + 2 * rz, SY = 2 * ry + 1, G = SY * (2 * rz + 1);
+    const int BY = RC_TY + 2 * ry, SY = 2 * ry + 1, G = SY * (2 * rz + 1);
     unsigned long long *red = rsm64;                                      // [G][KX]
     uint16_t *As = reinterpret_cast<uint16_t *>(rsm64 + ((size_t)G * KX + 1) / 2 * 2);  // [RC_TZ][RC_TY][RC_TX]
     uint16_t *Bs = As + RC_TX * RC_TY * RC_TZ;                            // [BZ][BY][BP]
@@ -99,6 +100,10 @@ __global__ void __launch_bounds__(RC_THREADS) k_reg_corr(const RegPair *__restri
     if ((long long)bi >= (long long)nbx * nby * nbz) return;
     const int ax0 = u0.x + (bi % nbx) * RC_TX, ay0 = u0.y + ((bi / nbx) % nby) * RC_TY;
     const int az0 = u0.z + (bi / (nbx * nby)) * RC_TZ;
+    // a sub-box at the region's end (all of them, for flat tiles) has fewer
+    // planes (3 x 3 tiles of 1024 x 1024 x 4: 0.64 ms for the call, 0.99 with the
+    // missing ones multiplied as zeros)
+    const int TZ = min(RC_TZ, u1.z - az0), ROWS = RC_TY * TZ, BZ = TZ + 2 * rz;
     if (threadIdx.x < 2) smax[threadIdx.x] = 0u;
     for (int i = threadIdx.x; i < G * KX; i += RC_THREADS) red[i] = 0ull;
     __syncthreads();
@@ -106,17 +111,17 @@ __global__ void __launch_bounds__(RC_THREADS) k_reg_corr(const RegPair *__restri
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int WARPS = RC_THREADS / 32, RB = 4;
     uint32_t ma = 0, mb = 0;
-    for (int r0 = warp; r0 < RC_TY * RC_TZ; r0 += WARPS * RB) {
+    for (int r0 = warp; r0 < ROWS; r0 += WARPS * RB) {
         uint32_t v[RB];
 #pragma unroll
         for (int k = 0; k < RB; ++k) {
             const int row = r0 + k * WARPS, x = ax0 + lane, y = ay0 + row % RC_TY, z = az0 + row / RC_TY;
-            v[k] = row < RC_TY * RC_TZ && x < u1.x && y < u1.y && z < u1.z ? A[((size_t)z * Y + y) * X + x] : 0u;
+            v[k] = row < ROWS && x < u1.x && y < u1.y && z < u1.z ? A[((size_t)z * Y + y) * X + x] : 0u;
         }
 #pragma unroll
         for (int k = 0; k < RB; ++k) {
             const int row = r0 + k * WARPS;
-            if (row < RC_TY * RC_TZ) As[row * RC_TX + lane] = (uint16_t)v[k];
+            if (row < ROWS) As[row * RC_TX + lane] = (uint16_t)v[k];
             ma = max(ma, v[k]);
         }
     }
@@ -158,7 +163,6 @@ __global__ void __launch_bounds__(RC_THREADS) k_reg_corr(const RegPair *__restri
         atomicMax(&smax[1], mb);
     }
     __syncthreads();
-    constexpr int ROWS = RC_TY * RC_TZ;
     const int C = G >= RC_THREADS ? 1 : min(ROWS, RC_THREADS / G);  // row chunks per shift group
     // rows whose products sum to less than 2^32: each of the RC_TX products
     // is at most smax[0] smax[1] (< 2^32)
@@ -236,9 +240,12 @@ RegCorrFn reg_corr_fn(int rx, std::integer_sequence<int, R...>) {
     return f;
 }
 
-// Sums of v and v^2 over one plane of a side's region U for every x-range (one
-// per x-shift) and y-range (one per y-shift): p1, p2[((z - u0.z) SY + syi) SX +
-// sxi].  Block (z, 2 pair + side).  Ranges move monotonically with the shift:
+// Sums of v and v^2 over one slab of rows of one plane of a side's region U for
+// every x-range (one per x-shift) and y-range (one per y-shift): p1, p2[(slab SY
+// + syi) SX + sxi] of the side's `per` slabs.  Block (slab, 2 pair + side); a
+// plane is `ns` consecutive slabs, one unless the planes are too few to fill the
+// GPU (two tiles of 4096 x 4096 x 1 with a tenth of overlap: the call takes 186
+// us, 715 with a block per plane), and planes start at z0.  Ranges move monotonically with the shift:
 // all of them share a core [clo, chi) in x and in y, and outside it lie at most
 // 2 rx columns on either side.  The rows of the y-core add up in registers, the
 // x-core per lane and the outer columns one per lane, and are reduced once per
@@ -251,6 +258,7 @@ constexpr int RP_THREADS = 256, RP_SY = 2 * SEG_REG_MAX_RXY + 1;
 constexpr int RP_COLS = 64;  // outer columns: 32 left, 32 right (2 rx <= 24 used)
 
 __global__ void __launch_bounds__(RP_THREADS) k_reg_plane(const RegPair *__restrict__ pairs, int X, int Y, int3 r,
+                                                          int z0, int ns, size_t per,
                                                           unsigned long long *__restrict__ p1,
                                                           unsigned long long *__restrict__ p2) {
     // sums of v and v^2: entry SY holds the y-core, entry syi the other rows
@@ -259,7 +267,10 @@ __global__ void __launch_bounds__(RP_THREADS) k_reg_plane(const RegPair *__restr
     const RegPair &P = pairs[blockIdx.y >> 1];
     const int side = blockIdx.y & 1;
     const int3 u0 = P.u0[side], u1 = P.u1[side], d0 = P.d0;
-    if (u1.x <= u0.x || u1.y <= u0.y || (int)blockIdx.x >= u1.z - u0.z) return;
+    const int z = u0.z + z0 + (int)blockIdx.x / ns;
+    if (u1.x <= u0.x || u1.y <= u0.y || z >= u1.z) return;
+    const int uy = u1.y - u0.y, sh = (uy + ns - 1) / ns;  // this block's rows: [ya, yb)
+    const int ya = u0.y + min((int)blockIdx.x % ns * sh, uy), yb = min(ya + sh, u1.y);
     const int SX = 2 * r.x + 1, SY = 2 * r.y + 1;
     const int lane = threadIdx.x & 31;
     for (int i = threadIdx.x; i < 2 * (RP_SY + 1); i += RP_THREADS) (&xc[0][0])[i] = 0ull;
@@ -268,23 +279,24 @@ __global__ void __launch_bounds__(RP_THREADS) k_reg_plane(const RegPair *__restr
     const Range yf = shared_range(d0.y - r.y, Y, side), yl = shared_range(d0.y + r.y, Y, side);
     int clo = max(xf.lo, xl.lo), chi = min(xf.hi, xl.hi);
     const int ylo = max(yf.lo, yl.lo), yhi = min(yf.hi, yl.hi);
-    if (clo >= chi) clo = chi = u1.x;  // no core: at most 4 rx columns, all left ones
+    if (clo >= chi) clo = chi = u1.x;  // no core: at most 2 rx columns, all left ones
     // this lane's outer columns: u0.x + lane before clo, and chi + lane
     const int xa = u0.x + lane, xr = chi + lane;
     __syncthreads();
-    const uint16_t *plane = P.tile[side] + (size_t)(u0.z + (int)blockIdx.x) * X * Y;
+    const uint16_t *plane = P.tile[side] + (size_t)z * X * Y;
     unsigned long long a1 = 0, a2 = 0, l1 = 0, l2 = 0, h1 = 0, h2 = 0;  // y-core
     constexpr int WARPS = RP_THREADS / 32, RB = 4;
     const int warp = threadIdx.x >> 5;
     // the y-core, RB rows' loads in flight
-    for (int y0 = ylo + warp; y0 < yhi; y0 += WARPS * RB) {
+    const int ye = min(yhi, yb);
+    for (int y0 = max(ylo, ya) + warp; y0 < ye; y0 += WARPS * RB) {
         const uint16_t *t[RB];
         bool on[RB];
         uint32_t va[RB], vr[RB];
 #pragma unroll
         for (int k = 0; k < RB; ++k) {
             const int y = y0 + k * WARPS;
-            on[k] = y < yhi;
+            on[k] = y < ye;
             t[k] = plane + (size_t)(on[k] ? y : y0) * X;
             va[k] = on[k] && xa < clo ? t[k][xa] : 0u;
             vr[k] = on[k] && xr < u1.x ? t[k][xr] : 0u;
@@ -308,9 +320,9 @@ __global__ void __launch_bounds__(RP_THREADS) k_reg_plane(const RegPair *__restr
         }
     }
     // the rows outside it
-    const int before = max(min(ylo, u1.y) - u0.y, 0), start = max(yhi, u0.y + before);
-    for (int i = warp; i < before + (u1.y - start); i += WARPS) {
-        const int y = i < before ? u0.y + i : start + (i - before);
+    const int before = max(min(ylo, yb) - ya, 0), start = max(yhi, ya + before);
+    for (int i = warp; i < before + max(yb - start, 0); i += WARPS) {
+        const int y = i < before ? ya + i : start + (i - before);
         const uint16_t *t = plane + (size_t)y * X;
         const uint32_t va = xa < clo ? t[xa] : 0u, vr = xr < u1.x ? t[xr] : 0u;
         unsigned long long s1 = 0, s2 = 0;
@@ -355,7 +367,7 @@ __global__ void __launch_bounds__(RP_THREADS) k_reg_plane(const RegPair *__restr
     atomicAdd(&col[0][SY][32 + lane], h1);
     atomicAdd(&col[1][SY][32 + lane], h2);
     __syncthreads();
-    const size_t o = P.planes[side] + (size_t)blockIdx.x * SY * SX;
+    const size_t o = per * blockIdx.y + (size_t)blockIdx.x * SY * SX;
     for (int i = threadIdx.x; i < SY * SX; i += RP_THREADS) {
         const int sy = i / SX;
         const Range wx = shared_range(d0.x + i % SX - r.x, X, side), wy = shared_range(d0.y + sy - r.y, Y, side);
@@ -373,27 +385,34 @@ __global__ void __launch_bounds__(RP_THREADS) k_reg_plane(const RegPair *__restr
 }
 
 // Per shift: the sums of v and v^2 over a side's shared box, one thread per
-// shift adding its planes; block (shifts, 2 pair + side).
+// shift adding the slabs of BOX_SLABS / ns planes from z0 on; block (shifts,
+// 2 pair + side, planes).  With all planes in one thread deep tiles waited for
+// it (two tiles of 16 x 16 x 20000: 5.7 ms for the call, now 0.92).
+constexpr int BOX_SLABS = 64;
+
 __global__ void k_reg_box(const RegPair *__restrict__ pairs, const unsigned long long *__restrict__ p1,
-                          const unsigned long long *__restrict__ p2, int X, int Y, int Z, int3 r,
-                          unsigned long long *__restrict__ sums, size_t per) {
+                          const unsigned long long *__restrict__ p2, int X, int Y, int Z, int3 r, int z0, int z1,
+                          int ns, size_t pper, unsigned long long *__restrict__ sums, size_t per) {
     const RegPair &P = pairs[blockIdx.y >> 1];
     const int side = blockIdx.y & 1;
     const int3 u0 = P.u0[side], u1 = P.u1[side], d0 = P.d0;
     const int SX = 2 * r.x + 1, SY = 2 * r.y + 1, S = SX * SY * (2 * r.z + 1);
     const int si = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    if (si >= S) return;
+    if (si >= S || u1.x <= u0.x || u1.y <= u0.y) return;
     const Range zr = shared_range(d0.z + si / (SX * SY) - r.z, Z, side);
+    const int nz = max(BOX_SLABS / ns, 1), za = z0 + (int)blockIdx.z * nz;  // planes from u0.z on
+    const int lo = max(zr.lo - u0.z, za), hi = min(zr.hi - u0.z, min(za + nz, z1));
+    if (lo >= hi) return;
     unsigned long long a = 0, b = 0;
-    if (u1.x > u0.x && u1.y > u0.y)
-        for (int z = zr.lo; z < zr.hi; ++z) {
-            const size_t i = P.planes[side] + (size_t)(z - u0.z) * SY * SX + si % (SX * SY);
-            a += p1[i];
-            b += p2[i];
-        }
+    const size_t at = pper * blockIdx.y + si % (SX * SY);
+    for (int q = (lo - z0) * ns; q < (hi - z0) * ns; ++q) {
+        const size_t i = at + (size_t)q * SY * SX;
+        a += p1[i];
+        b += p2[i];
+    }
     unsigned long long *o = sums + per * (blockIdx.y >> 1) + (size_t)(1 + 2 * side) * S;
-    o[si] = a;
-    o[S + si] = b;
+    if (a) atomicAdd(o + si, a);
+    if (b) atomicAdd(o + S + si, b);
 }
 
 int fail(cudaError_t e) {
@@ -526,25 +545,45 @@ extern "C" int seg_register_montage(int device, const uint16_t *const *tiles, in
     unsigned long long *dsum, *dp1, *dp2;
     RegPair *dpair;
     std::vector<RegPair> pairs(E.size());
-    size_t npl = 1;  // plane sums of the largest group
-    for (size_t ei = 0, used = 0; ei < E.size(); ++ei) {
+    int most_y = 0, most_z = 0;  // rows and planes of the largest search regions, voxels of a plane
+    size_t most_xy = 0;
+    for (size_t ei = 0; ei < E.size(); ++ei) {
         const seg_montage_edge &e = E[ei];
         RegPair &P = pairs[ei];
-        if (ei % REG_GROUP == 0) used = 0;
         const int d0[3] = {stage[e.b].x - stage[e.a].x, stage[e.b].y - stage[e.a].y, stage[e.b].z - stage[e.a].z};
         P.tile[0] = dt[e.a];
         P.tile[1] = dt[e.b];
         P.d0 = make_int3(d0[0], d0[1], d0[2]);
         for (int side = 0; side < 2; ++side) {
             side_region(d0, r, D, side, P.u0[side], P.u1[side]);
-            P.planes[side] = used;
-            used += (size_t)SX * SY * (size_t)(P.u1[side].z - P.u0[side].z);
+            const int uy = P.u1[side].y - P.u0[side].y;
+            most_xy = std::max(most_xy, (size_t)uy * (P.u1[side].x - P.u0[side].x));
+            most_y = std::max(most_y, uy);
+            most_z = std::max(most_z, P.u1[side].z - P.u0[side].z);
         }
-        npl = std::max(npl, used);
     }
+    // Planes are cut into slabs while a group has fewer than PLANE_BLOCKS of
+    // them per multiprocessor, down to SLAB_ROWS rows and SLAB_VOXELS voxels
+    // (slabs of 40 rows of 20 voxels cost 10 % of a call that takes 132 us with
+    // whole planes), and taken PZ at a time so that their sums stay within
+    // PLANE_BYTES (a single plane of every pair: at most 82 MB, for 64 pairs, 64
+    // slabs and 25 x 25 shifts).
+    constexpr int SLAB_ROWS = 32, PLANE_BLOCKS = 4, MAX_SLABS = 64;
+    constexpr size_t SLAB_VOXELS = 16384, PLANE_BYTES = 256u << 20;
+    int sms = 0;
+    RK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
+    int ns = 1;
+    while (ns < MAX_SLABS && 2 * ns * SLAB_ROWS <= most_y && 2 * ns * SLAB_VOXELS <= most_xy &&
+           2 * gmax * most_z * ns < (size_t)PLANE_BLOCKS * sms)
+        ns *= 2;
+    const size_t plane = (size_t)SX * SY * ns;  // sums of one plane of one side
+    const int PZ = (int)std::max<size_t>(
+        1, std::min<size_t>(std::min<size_t>((size_t)most_z, 65535),  // (the last grid dimension of k_reg_box)
+                            PLANE_BYTES / (2 * sizeof(unsigned long long) * 2 * gmax * plane)));
+    const size_t pper = plane * PZ;
     RK(sc.alloc(&dsum, per * gmax));
-    RK(sc.alloc(&dp1, npl));
-    RK(sc.alloc(&dp2, npl));
+    RK(sc.alloc(&dp1, 2 * gmax * pper));
+    RK(sc.alloc(&dp2, 2 * gmax * pper));
     RK(sc.alloc(&dpair, gmax));
     std::vector<unsigned long long> hs(per * gmax);
     const size_t smem = reg_corr_smem(r[0], r[1], r[2]);
@@ -566,10 +605,12 @@ extern "C" int seg_register_montage(int device, const uint16_t *const *tiles, in
         }
         RK(cudaMemcpyAsync(dpair, pairs.data() + g0, ng * sizeof(RegPair), cudaMemcpyHostToDevice, sc.s));
         RK(cudaMemsetAsync(dsum, 0, per * ng * sizeof(unsigned long long), sc.s));
-        if (nz > 0) {
-            k_reg_plane<<<dim3((unsigned)nz, 2 * ng), RP_THREADS, 0, sc.s>>>(dpair, D[0], D[1], r3, dp1, dp2);
-            k_reg_box<<<dim3((unsigned)((S + 63) / 64), 2 * ng), 64, 0, sc.s>>>(dpair, dp1, dp2, D[0], D[1], D[2], r3,
-                                                                               dsum, per);
+        for (int z0 = 0; z0 < nz; z0 += PZ) {
+            const int n = std::min(PZ, nz - z0), bz = std::max(BOX_SLABS / ns, 1);
+            k_reg_plane<<<dim3((unsigned)(n * ns), 2 * ng), RP_THREADS, 0, sc.s>>>(dpair, D[0], D[1], r3, z0, ns, pper,
+                                                                                   dp1, dp2);
+            k_reg_box<<<dim3((unsigned)((S + 63) / 64), 2 * ng, (unsigned)((n + bz - 1) / bz)), 64, 0, sc.s>>>(
+                dpair, dp1, dp2, D[0], D[1], D[2], r3, z0, z0 + n, ns, pper, dsum, per);
         }
         if (nb > 0)
             corr<<<dim3((unsigned)nb, ng), RC_THREADS, smem, sc.s>>>(dpair, D[0], D[1], D[2], r[1], r[2], dsum, per);
