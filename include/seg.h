@@ -371,7 +371,8 @@ typedef struct {
  * position; 0 for tiles the tree does not reach).  edges (cap edges_cap)
  * gets the pairs in (a, b) order and *n_edges their number.  Blocks until
  * done.  Errors: SEG_EINVAL (null pointer, zero size, root >= n_tiles, a
- * radius outside its limit), SEG_ETOOBIG (a tile of 2^32 voxels or more),
+ * radius outside its limit), SEG_ETOOBIG (a tile of 2^32 voxels or more, or
+ * longer than SEG_MAX_YZ along an axis),
  * SEG_ESMALL (edges_cap < *n_edges: nothing else is written), SEG_ECUDA. */
 int seg_register_montage(int device, const uint16_t *const *tiles, int on_device, uint32_t n_tiles,
                          seg_dims dims, const seg_offset *stage, seg_offset radius, uint32_t root,

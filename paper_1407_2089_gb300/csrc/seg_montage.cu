@@ -46,10 +46,11 @@ struct Range {
 };
 
 // Shared range along one axis for tile b's origin at d in tile a's frame:
-// in a's coordinates (side 0) or in b's (side 1).
+// in a's coordinates (side 0) or in b's (side 1).  d + D and D - d are only
+// formed where they are at most D, so that no tile extent overflows them.
 __host__ __device__ inline Range shared_range(int d, int D, int side) {
-    if (side == 0) return Range{d > 0 ? d : 0, d + D < D ? d + D : D};
-    return Range{-d > 0 ? -d : 0, D - d < D ? D - d : D};
+    if (side == 0) return Range{d > 0 ? d : 0, d < 0 ? d + D : D};
+    return Range{d < 0 ? -d : 0, d > 0 ? D - d : D};
 }
 
 // One overlapping pair on the device: tile b's origin in tile a's frame, the
@@ -487,8 +488,8 @@ extern "C" int seg_register_montage(int device, const uint16_t *const *tiles, in
     for (uint32_t i = 0; i < n_tiles; ++i)
         if (!tiles[i]) return SEG_EINVAL;
     const uint64_t n = (uint64_t)dims.x * dims.y * dims.z;
-    if (n >= (1ull << 32) || dims.x > 0x7FFFFFFFu || dims.y > 0x7FFFFFFFu || dims.z > 0x7FFFFFFFu)
-        return SEG_ETOOBIG;
+    // the kernels step up to 63 positions past a tile's end in signed integers
+    if (n >= (1ull << 32) || dims.x > SEG_MAX_YZ || dims.y > SEG_MAX_YZ || dims.z > SEG_MAX_YZ) return SEG_ETOOBIG;
     const int D[3] = {(int)dims.x, (int)dims.y, (int)dims.z};
     const int r[3] = {radius.x, radius.y, radius.z};
     // pairs whose stage boxes overlap, in (a, b) order
