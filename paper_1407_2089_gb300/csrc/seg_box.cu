@@ -2,7 +2,8 @@
 // Removal, Eq. 1): three rounded box passes of radius r along x, then y, then
 // z, each pass with replicate edges.
 //
-// One thread follows one line (or a chunk of one) and runs all three passes at
+// Two forms, chosen per axis (box_rings()).  In register rings one thread
+// follows one line (or a chunk of one) and runs all three passes at
 // once: position p of the input feeds the first running sum, whose value at
 // p - r feeds the second, whose value at p - 2r feeds the third, which gives
 // the output at p - 3r.  The 2r + 1 values in each window stay in registers as
@@ -16,10 +17,12 @@
 // of them; a chunk inside a line starts 3r positions early with empty rings,
 // which fill by the time its first output is due.
 //
-// Bound by instruction issue.  4 volumes of 512 x 512 x 64, r = 8: x 238 -> 223,
-// y 154 -> 101, z 214 -> 148 us against three passes through shared memory with a
-// barrier each.  Chunks of 256 positions along x (two blocks fewer resident) take
-// 330 us there.
+// Bound by the latency of its loads along x and y (IPC 1.6 and 1.8 of 4, long
+// scoreboard first), between that and instruction issue along z (2.2).  4 volumes
+// of 512 x 512 x 64, r = 8: x 238 -> 223, y 153 -> 101, z 214 -> 147 us against the
+// other form, three passes through shared memory with a barrier each (k_box3),
+// which is the faster one for small batches and large radii.  Chunks of 256
+// positions along x (two blocks fewer resident) take 330 us there.
 #include <algorithm>
 #include <cstdint>
 
@@ -148,8 +151,6 @@ __device__ __forceinline__ void box_line_r(int r, const uint16_t *src, uint16_t 
 #undef SEG_BOX_R
 }
 
-__device__ __forceinline__ int box_class(uint32_t r) { return r <= 4 ? 0 : (r <= 8 ? 1 : 2); }
-
 template <int AXIS>
 __device__ __forceinline__ uint32_t box_base(const VolDev &V) {
     return AXIS == 0 ? V.dn_base0 : (AXIS == 1 ? V.dn_base1 : V.dn_base2);
@@ -173,7 +174,7 @@ template <int AXIS, int CLS>
 __global__ void __launch_bounds__(BX_THREADS) k_box_lines(const BatchHdr *__restrict__ h) {
     for (uint32_t it = blockIdx.x; it < h->dn_items[AXIS]; it += gridDim.x) {
         const VolDev &V = h->vol[box_volume<AXIS>(h, it)];
-        if (box_class(V.dn_r) != CLS) continue;
+        if (box_class(V.dn_r) != CLS || !(V.dn_ring >> AXIS & 1u)) continue;
         const uint32_t li = it - box_base<AXIS>(V);
         const uint32_t len = AXIS == 1 ? V.Y : V.Z, nchunk = box_chunks(len, DN_CHUNK);
         const BoxChunk c = box_chunk(len, DN_CHUNK, li % nchunk, V.dn_r);
@@ -200,7 +201,7 @@ __global__ void __launch_bounds__(BX_THREADS) k_box_x(const BatchHdr *__restrict
     constexpr int WARPS = BX_THREADS / 32, RB = 8;
     for (uint32_t it = blockIdx.x; it < h->dn_items[0]; it += gridDim.x) {
         const VolDev &V = h->vol[box_volume<0>(h, it)];
-        if (box_class(V.dn_r) != CLS) continue;
+        if (box_class(V.dn_r) != CLS || !(V.dn_ring & 1u)) continue;
         const uint32_t li = it - V.dn_base0;
         const int n = (int)V.X, r = (int)V.dn_r, nchunk = (n + DN_CHUNK_X - 1) / DN_CHUNK_X;
         const int per = (n + nchunk - 1) / nchunk;
@@ -243,34 +244,262 @@ __global__ void __launch_bounds__(BX_THREADS) k_box_x(const BatchHdr *__restrict
     }
 }
 
-template <int CLS>
-void launch_class(const BatchHdr *d, const LaunchPlan &p, cudaStream_t s) {
-    k_box_x<CLS><<<p.grid_box, BX_THREADS, box_x_smem(CLS == 0 ? 4 : (CLS == 1 ? 8 : 16)), s>>>(d);
-    k_box_lines<1, CLS><<<p.grid_box, BX_THREADS, 0, s>>>(d);
-    k_box_lines<2, CLS><<<p.grid_box, BX_THREADS, 0, s>>>(d);
+// The same passes through shared memory, for small batches and large radii
+// (box_rings()): an item is 64 lines x a chunk of at most BOX_CHUNK positions,
+// loaded with a halo of 3r positions on each side; pass k runs over the
+// positions the next one needs, four threads per line, each reading its input at
+// positions clamped to the line, which is the replicate edge of every pass.
+// Four times the threads per voxel of the register rings, and registers that do
+// not grow with r.  Shared layout [position][lane], lanes padded to 66 so that
+// both the lane-major passes and the position-major copies of axis x avoid bank
+// conflicts.
+constexpr int BOX_THREADS = 256, BOX_CHUNK = 128;
+constexpr int BOX_LANES = 64, BOX_PITCH = BOX_LANES + 2;
+constexpr int BOX_POS = BOX_CHUNK + 6 * DN_MAX_R;
+constexpr size_t BOX_SMEM = 2ull * BOX_POS * BOX_PITCH * sizeof(uint16_t);
+
+template <int AXIS>
+__global__ void __launch_bounds__(BOX_THREADS) k_box3(const BatchHdr *__restrict__ h) {
+    extern __shared__ __align__(16) uint16_t bsm[];
+    uint16_t *bufA = bsm, *bufB = bsm + BOX_POS * BOX_PITCH;
+    const int t = threadIdx.x;
+    for (uint32_t it = blockIdx.x; it < h->dn_items[AXIS]; it += gridDim.x) {
+        const VolDev &V = h->vol[box_volume<AXIS>(h, it)];
+        if (V.dn_ring >> AXIS & 1u) continue;
+        const uint32_t li = it - box_base<AXIS>(V), X = V.X;
+        const uint32_t len = AXIS == 0 ? X : (AXIS == 1 ? V.Y : V.Z), nchunk = box_chunks(len, BOX_CHUNK);
+        const uint32_t group = li / nchunk;
+        const int r = (int)V.dn_r;
+        const uint32_t mul = V.dn_mul;
+        const BoxChunk c = box_chunk(len, BOX_CHUNK, li % nchunk, V.dn_r);
+        const int n = c.n, c0 = c.c0, c1 = c.c1;
+        if (c0 >= c1) continue;  // (the same in every thread)
+        const int base = c0 - 3 * r, lo = 0, hi = min(c1 + 3 * r, n);  // loaded: [lo, hi)
+        // lane l of this group: its line's position 0 and the step along it
+        int nl;            // lanes of this group that exist
+        size_t gstart;     // element of lane 0 at position 0
+        size_t lstride, pstride;
+        if (AXIS == 0) {
+            nl = (int)min((uint32_t)BOX_LANES, V.rows - group * BOX_LANES);
+            gstart = (size_t)group * BOX_LANES * X;
+            lstride = X;
+            pstride = 1;
+        } else {
+            const uint32_t nxg = (X + BOX_LANES - 1) / BOX_LANES, gx = group % nxg, other = group / nxg;
+            nl = (int)min((uint32_t)BOX_LANES, X - gx * BOX_LANES);
+            lstride = 1;
+            if (AXIS == 1) {
+                gstart = (size_t)gx * BOX_LANES + (size_t)X * V.Y * other;
+                pstride = X;
+            } else {
+                gstart = (size_t)gx * BOX_LANES + (size_t)X * other;
+                pstride = (size_t)X * V.Y;
+            }
+        }
+        gstart += c.first * pstride;
+        const uint16_t *src = AXIS == 0 ? V.dn_src : (AXIS == 1 ? V.dn_a : V.dn_b);
+        uint16_t *dst = AXIS == 1 ? V.dn_b : V.dn_a;
+        const int np = hi - lo;
+        __syncthreads();  // the previous item is done with the buffers
+        // load: consecutive threads on consecutive elements in memory, eight
+        // independent loads in flight per thread before the shared stores
+        constexpr int NB = 8;
+        if (AXIS == 0) {
+            // one warp per line (a row segment), lanes along it
+            const int lane = t & 31, warp = t >> 5, nw = blockDim.x >> 5;
+            for (int l = warp; l < nl; l += nw) {
+                const uint16_t *row = src + gstart + (size_t)l * lstride;
+                for (int q0 = lo + lane; q0 < hi; q0 += 32 * NB) {
+                    uint16_t v[NB];
+#pragma unroll
+                    for (int j = 0; j < NB; ++j)
+                        if (q0 + 32 * j < hi) v[j] = row[q0 + 32 * j];
+#pragma unroll
+                    for (int j = 0; j < NB; ++j)
+                        if (q0 + 32 * j < hi) bufA[(q0 + 32 * j - base) * BOX_PITCH + l] = v[j];
+                }
+            }
+        } else if ((X & 7u) == 0u) {
+            // rows of 8-voxel octets (X % 8 == 0, scratch buffers 16-byte
+            // aligned): thread t moves lanes 8 (t % 8) .. + 7 of positions
+            // t / 8 + 32 i as one 16-byte load and four 4-byte shared stores
+            // (pitch 66: the 32 threads of a warp hit 32 different banks)
+            const int oct = t & 7, pr = t >> 3;
+            constexpr int NV = 4;
+            if (8 * oct < nl) {
+                const uint16_t *col = src + gstart + 8 * oct;
+                for (int q0 = lo + pr; q0 < hi; q0 += 32 * NV) {
+                    uint4 v[NV];
+#pragma unroll
+                    for (int j = 0; j < NV; ++j)
+                        if (q0 + 32 * j < hi)
+                            v[j] = *reinterpret_cast<const uint4 *>(col + (size_t)(q0 + 32 * j) * pstride);
+#pragma unroll
+                    for (int j = 0; j < NV; ++j)
+                        if (q0 + 32 * j < hi) {
+                            uint32_t *w = reinterpret_cast<uint32_t *>(bufA + (q0 + 32 * j - base) * BOX_PITCH + 8 * oct);
+                            w[0] = v[j].x; w[1] = v[j].y; w[2] = v[j].z; w[3] = v[j].w;
+                        }
+                }
+            }
+        } else {
+            const int total = np * BOX_LANES, nt = blockDim.x;
+            for (int i0 = t; i0 < total; i0 += nt * NB) {
+                uint16_t v[NB];
+#pragma unroll
+                for (int j = 0; j < NB; ++j) {
+                    const int i = i0 + j * nt, l = i % BOX_LANES, q = lo + i / BOX_LANES;
+                    if (i < total && l < nl) v[j] = src[gstart + (size_t)l * lstride + (size_t)q * pstride];
+                }
+#pragma unroll
+                for (int j = 0; j < NB; ++j) {
+                    const int i = i0 + j * nt, l = i % BOX_LANES, q = lo + i / BOX_LANES;
+                    if (i < total && l < nl) bufA[(q - base) * BOX_PITCH + l] = v[j];
+                }
+            }
+        }
+        __syncthreads();
+        // three passes: A -> B over [c0-2r, c1+2r), B -> A over [c0-r, c1+r), A -> B over [c0, c1)
+        const int l = t % BOX_LANES, seg = t / BOX_LANES;
+        for (int k = 0; k < 3; ++k) {
+            const uint16_t *in = (k == 1) ? bufB : bufA;
+            uint16_t *out = (k == 1) ? bufA : bufB;
+            const int p0 = max(c0 - (2 - k) * r, 0), p1 = min(c1 + (2 - k) * r, n);
+            const int per = (p1 - p0 + 3) / 4;
+            const int q0 = p0 + seg * per, q1 = min(q0 + per, p1);
+            if (l < nl && q0 < q1) {
+                // every read lies in [q0 - r, q1 - 1 + r] clamped to the line,
+                // inside the positions the previous pass (or the load) covered
+                auto at = [&](int q) { return (uint32_t)in[(min(max(q, 0), n - 1) - base) * BOX_PITCH + l]; };
+                // sum holds the window sum plus the rounding term r
+                uint32_t sum = (uint32_t)r;
+                if (q0 - r >= 0 && q0 + r < n) {
+                    const uint16_t *pw = in + (q0 - r - base) * BOX_PITCH + l;
+                    for (int i = 0; i <= 2 * r; ++i) sum += pw[i * BOX_PITCH];
+                } else {
+                    for (int q = q0 - r; q <= q0 + r; ++q) sum += at(q);
+                }
+                out[(q0 - base) * BOX_PITCH + l] = (uint16_t)box_div(sum, mul);
+                // positions q whose window [q - r - 1, q + r] needs no
+                // clamping run through three moving pointers
+                const int qa = min(max(q0 + 1, r + 1), q1), qb = max(min(q1, n - r), qa);
+                int q = q0 + 1;
+                for (; q < qa; ++q) {
+                    sum += at(q + r) - at(q - r - 1);
+                    out[(q - base) * BOX_PITCH + l] = (uint16_t)box_div(sum, mul);
+                }
+                const uint16_t *pin = in + (q + r - base) * BOX_PITCH + l;
+                const uint16_t *pout = in + (q - r - 1 - base) * BOX_PITCH + l;
+                uint16_t *po = out + (q - base) * BOX_PITCH + l;
+#pragma unroll 4
+                for (; q < qb; ++q) {
+                    sum += (uint32_t)*pin - (uint32_t)*pout;
+                    *po = (uint16_t)box_div(sum, mul);
+                    pin += BOX_PITCH;
+                    pout += BOX_PITCH;
+                    po += BOX_PITCH;
+                }
+                for (; q < q1; ++q) {
+                    sum += at(q + r) - at(q - r - 1);
+                    out[(q - base) * BOX_PITCH + l] = (uint16_t)box_div(sum, mul);
+                }
+            }
+            __syncthreads();
+        }
+        // store the chunk from B
+        const int nc = c1 - c0;
+        if (AXIS == 0) {
+            const int lane = t & 31, warp = t >> 5, nw = blockDim.x >> 5;
+            for (int ll = warp; ll < nl; ll += nw) {
+                uint16_t *row = dst + gstart + (size_t)ll * lstride;
+                for (int q = c0 + lane; q < c1; q += 32) row[q] = bufB[(q - base) * BOX_PITCH + ll];
+            }
+        } else if ((X & 7u) == 0u) {
+            const int oct = t & 7, pr = t >> 3;
+            if (8 * oct < nl) {
+                uint16_t *col = dst + gstart + 8 * oct;
+                for (int q = c0 + pr; q < c1; q += 32) {
+                    const uint32_t *w = reinterpret_cast<const uint32_t *>(bufB + (q - base) * BOX_PITCH + 8 * oct);
+                    *reinterpret_cast<uint4 *>(col + (size_t)q * pstride) = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            }
+        } else {
+            for (int i = t; i < nc * BOX_LANES; i += blockDim.x) {
+                const int ll = i % BOX_LANES, q = c0 + i / BOX_LANES;
+                if (ll < nl) dst[gstart + (size_t)ll * lstride + (size_t)q * pstride] = bufB[(q - base) * BOX_PITCH + ll];
+            }
+        }
+    }
 }
 
 }  // namespace
 
-uint32_t box_lines_items(uint64_t lines, uint32_t n, uint32_t chunk) {
-    return (uint32_t)((lines + BX_THREADS - 1) / BX_THREADS * box_chunks(n, chunk));
+uint64_t box_items(int axis, bool ring, uint32_t X, uint32_t Y, uint32_t Z) {
+    const uint32_t n = axis == 0 ? X : (axis == 1 ? Y : Z);
+    if (ring) {
+        const uint64_t lines = axis == 0 ? (uint64_t)Y * Z : (uint64_t)X * (axis == 1 ? Z : Y);
+        return (lines + BX_THREADS - 1) / BX_THREADS * box_chunks(n, axis == 0 ? DN_CHUNK_X : DN_CHUNK);
+    }
+    const uint64_t groups = axis == 0 ? ((uint64_t)Y * Z + BOX_LANES - 1) / BOX_LANES
+                                      : (uint64_t)((X + BOX_LANES - 1) / BOX_LANES) * (axis == 1 ? Z : Y);
+    return groups * box_chunks(n, BOX_CHUNK);
 }
 
-cudaError_t configure_box() {
-    const void *fn[3] = {(const void *)k_box_x<0>, (const void *)k_box_x<1>, (const void *)k_box_x<2>};
-    const int r[3] = {4, 8, 16};
-    for (int k = 0; k < 3; ++k) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(fn[k], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)box_x_smem(r[k]));
-        if (e != cudaSuccess) return e;
-    }
+// Where the rings are the faster ones, from both timed per axis for radii 1..16
+// on 40 batches (64 x 64 x 12 to 2000 x 2000 x 16).  They need enough lines (a
+// thread each; 128 x 128 x 32 at r = 8: 17.2 us along x and 8.1 along y, 10.2 and
+// 6.7 through shared memory), registers for the windows (above r = 8 two or three
+// blocks are resident: 512 x 512 x 64 at r = 12, x 130 against 68 us) and are
+// worth most where the shared copies of lines across rows are narrow (X % 8 != 0)
+// or the halo is long against the line (small Z):
+//   x: up to r = 8, for rows of one chunk (64 x 64 x 2000: 36 against 47 us) and
+//      large batches of whole chunks or small radii (four 512 x 512 x 64 volumes,
+//      r = 8: 223 against 238; not 700 x 700 x 80 at r = 8: 178 against 152);
+//   y: whole octets from r = 3 (few loads in flight below: r = 1 takes 1.3 times
+//      the time) to 8 (four 512 x 512 x 64 volumes: 101 against 153); ragged rows
+//      at any radius (511 x 511 x 64, r = 12: 39 against 70);
+//   z: up to r = 8 (147 against 214), above it for ragged rows and few planes
+//      (512 x 512 x 12, r = 10: 26 against 38; not 512 x 512 x 64 at r = 16: 81
+//      against 63).
+uint32_t box_rings(uint32_t X, uint32_t Z, uint32_t r, const uint64_t *items, int sms) {
+    const double S = (double)sms, x = (double)items[0] / S, y = (double)items[1] / S, z = (double)items[2] / S;
+    const bool octets = X % 8u == 0u;
+    uint32_t m = 0;
+    if (r <= 8u && (X <= 64u ? x >= 3.0 : (r <= 4u || X % 128u == 0u) && x >= 16.0)) m |= 1u;
+    if (octets ? r >= 2u && r <= 8u && y >= (r == 2u ? 3.0 : 2.5) : y >= (r == 1u ? 2.5 : (r == 2u ? 1.25 : 0.75))) m |= 2u;
+    if (z >= 2.0 && (r <= 8u || !octets || (r <= 12u && Z <= 32u))) m |= 4u;
+    return m;
+}
+
+cudaError_t configure_box(LaunchPlan &plan) {
+    const void *fn[5] = {(const void *)k_box_x<0>, (const void *)k_box_x<1>, (const void *)k_box3<0>,
+                         (const void *)k_box3<1>, (const void *)k_box3<2>};
+    const size_t smem[5] = {box_x_smem(4), box_x_smem(8), BOX_SMEM, BOX_SMEM, BOX_SMEM};
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < 5 && e == cudaSuccess; ++k)
+        e = cudaFuncSetAttribute(fn[k], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem[k]);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_box3<1>, BOX_THREADS, BOX_SMEM)) != cudaSuccess)
+        return e;
+    plan.grid_box3 = plan.sms * (per_sm > 0 ? per_sm : 1);
+    plan.grid_box = 16 * plan.sms;  // every ring kernel's resident blocks, at most
     return cudaSuccess;
 }
 
 void launch_box_passes(const BatchHdr *d, const LaunchPlan &p, cudaStream_t s) {
-    if (p.denoise & 1u) launch_class<0>(d, p, s);
-    if (p.denoise & 2u) launch_class<1>(d, p, s);
-    if (p.denoise & 4u) launch_class<2>(d, p, s);
+    auto on = [&](int axis, int route) { return (p.denoise >> box_route_bit(axis, route) & 1u) != 0u; };
+    if (on(0, 0)) k_box_x<0><<<p.grid_box, BX_THREADS, box_x_smem(4), s>>>(d);
+    if (on(0, 1)) k_box_x<1><<<p.grid_box, BX_THREADS, box_x_smem(8), s>>>(d);
+    if (on(0, 3)) k_box3<0><<<p.grid_box3, BOX_THREADS, BOX_SMEM, s>>>(d);
+    if (on(1, 0)) k_box_lines<1, 0><<<p.grid_box, BX_THREADS, 0, s>>>(d);
+    if (on(1, 1)) k_box_lines<1, 1><<<p.grid_box, BX_THREADS, 0, s>>>(d);
+    if (on(1, 2)) k_box_lines<1, 2><<<p.grid_box, BX_THREADS, 0, s>>>(d);
+    if (on(1, 3)) k_box3<1><<<p.grid_box3, BOX_THREADS, BOX_SMEM, s>>>(d);
+    if (on(2, 0)) k_box_lines<2, 0><<<p.grid_box, BX_THREADS, 0, s>>>(d);
+    if (on(2, 1)) k_box_lines<2, 1><<<p.grid_box, BX_THREADS, 0, s>>>(d);
+    if (on(2, 2)) k_box_lines<2, 2><<<p.grid_box, BX_THREADS, 0, s>>>(d);
+    if (on(2, 3)) k_box3<2><<<p.grid_box3, BOX_THREADS, BOX_SMEM, s>>>(d);
 }
 
 }  // namespace seg

@@ -106,6 +106,7 @@ struct VolDev {
     uint16_t *dn_out;         // denoised image (the smoothing's input)
     uint32_t dn_r;            // box radius, 0 = no denoise
     uint32_t dn_mul;          // ceil(2^32 / (2 dn_r + 1)): division by the box width
+    uint32_t dn_ring;         // bit a: axis a by register rings (box_rings())
     uint32_t dn_n[3];         // box-pass items per axis (groups of lines x chunks)
     uint32_t dn_base0, dn_base1, dn_base2;  // first flat box item per axis
     uint32_t dn_tiles;        // median tiles
@@ -199,10 +200,11 @@ struct LaunchPlan {
     int grid_task;       // k_union, k_flatten
     int grid_lab;        // k_label_features
     int grid_box;        // k_box_x, k_box_lines
+    int grid_box3;       // k_box3
     int grid_med;        // k_median27
     bool rows;           // some volume of the batch takes k_smooth_rows
     bool tiles;          // some volume of the batch takes k_smooth_hist
-    uint32_t denoise;    // denoise front end: bit k set for volumes of radius class k (1..4, 5..8, 9..16)
+    uint32_t denoise;    // denoise front end: box_route_bit()s of its volumes (0: none)
     bool closing;        // some volume of the batch closes its foreground
     bool distance;       // some volume of the batch has a distance map
     int grid_dist;       // k_dist_x, k_dist_line
@@ -252,10 +254,18 @@ __host__ __device__ inline BoxChunk box_chunk(uint32_t n, uint32_t chunk, uint32
     const uint32_t lead = at < 3u * r ? at : 3u * r, len = n - at < per ? n - at : per;
     return BoxChunk{at - lead, (int)(n - (at - lead)), (int)lead, (int)(lead + len), at == lead};
 }
-// Box passes (seg_box.cu): items of one axis for `lines` lines of n positions,
-// kernel attributes, and the launches.
-uint32_t box_lines_items(uint64_t lines, uint32_t n, uint32_t chunk);
-cudaError_t configure_box();
+// Box passes (seg_box.cu).  Route of a volume along an axis: 0, 1 or 2, the
+// register rings of its radius class (1..4, 5..8, 9..16), or 3, the passes
+// through shared memory; LaunchPlan::denoise has a bit per axis and route.
+__host__ __device__ inline int box_class(uint32_t r) { return r <= 4u ? 0 : (r <= 8u ? 1 : 2); }
+inline int box_route_bit(int axis, int route) { return 4 * axis + route; }
+// Work items of one axis of one volume, by either route.
+uint64_t box_items(int axis, bool ring, uint32_t X, uint32_t Y, uint32_t Z);
+// The axes (bit 0: x, 1: y, 2: z) along which a volume takes the rings; items:
+// the batch's items per axis, were all its volumes to take them.
+uint32_t box_rings(uint32_t X, uint32_t Z, uint32_t r, const uint64_t *items, int sms);
+// Kernel attributes and the grids of `plan`, and the launches.
+cudaError_t configure_box(LaunchPlan &plan);
 void launch_box_passes(const BatchHdr *d, const LaunchPlan &plan, cudaStream_t s);
 
 // Cell-to-vessel distance: out[k - 1] = min of map over the voxels labelled k.

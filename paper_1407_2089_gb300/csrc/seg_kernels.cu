@@ -4147,8 +4147,7 @@ cudaError_t configure_kernels(int device, LaunchPlan &plan) {
     if ((e = resident((const void *)k_flatten, ROW_TILE, &g2)) != cudaSuccess) return e;
     plan.grid_task = std::min(g1, g2);
     if ((e = resident((const void *)k_label_features, ROW_TILE, &plan.grid_lab)) != cudaSuccess) return e;
-    if ((e = configure_box()) != cudaSuccess) return e;
-    plan.grid_box = 16 * plan.sms;  // every class's resident blocks, at most
+    if ((e = configure_box(plan)) != cudaSuccess) return e;
     if ((e = resident((const void *)k_median27, MED_TX * MED_TY, &plan.grid_med)) != cudaSuccess) return e;
     if ((e = resident((const void *)k_dist_x, 256, &g1)) != cudaSuccess) return e;
     if ((e = resident((const void *)k_dist_line<2>, 256, &g2)) != cudaSuccess) return e;

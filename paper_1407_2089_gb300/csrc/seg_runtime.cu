@@ -182,7 +182,7 @@ struct Batch {
     uint32_t nvol = 0;
     uint64_t voxels = 0;
     uint32_t mrf_iters = 0;  // MRF steps launched (the largest limit in the batch)
-    uint32_t dn_classes = 0; // radius classes of the denoise front end in the batch
+    uint32_t dn_routes = 0;  // box-pass routes of the denoise front end in the batch
     std::atomic<bool> done{false};
     int launch_err = SEG_OK;
     struct seg_ctx *ctx = nullptr;
@@ -410,10 +410,15 @@ void build_header(seg_ctx *ctx, Batch &b) {
     const uint32_t rtile = batch_row_tile(ctx, b), lbk = batch_label_shrink(ctx, b);
     const uint64_t bkv = batch_brick_voxels(ctx, b);
     uint32_t fst = 0, lbs = 0;
-    uint32_t v = 0, tiles = 0, rts = 0, bks = 0, bts = 0, dn[3] = {0, 0, 0}, dnt = 0, cl = 0, dn_classes = 0;
+    uint32_t v = 0, tiles = 0, rts = 0, bks = 0, bts = 0, dn[3] = {0, 0, 0}, dnt = 0, cl = 0, dn_routes = 0;
     uint32_t dtb[DT_NK] = {0, 0, 0, 0, 0, 0};
     uint32_t mrft = 0, mrf_iters = 0;
     uint64_t mrfu = 0;
+    uint64_t dn_all[3] = {0, 0, 0};  // box-pass items per axis, were all by register rings
+    for (const Request *r : b.reqs)
+        for (const VolGeom &g : r->g)
+            if (g.dn_r)
+                for (int a = 0; a < 3; ++a) dn_all[a] += box_items(a, true, g.X, g.Y, g.Z);
     char *sp = b.scratch;
     for (Request *r : b.reqs) {
         for (uint32_t c = 0; c < r->C; ++c) {
@@ -427,7 +432,7 @@ void build_header(seg_ctx *ctx, Batch &b) {
             V.dn_src = V.raw;
             V.dn_a = V.dn_b = V.dn_out = nullptr;
             V.dn_mul = 0;
-            V.dn_n[0] = V.dn_n[1] = V.dn_n[2] = 0;
+            V.dn_ring = V.dn_n[0] = V.dn_n[1] = V.dn_n[2] = 0;
             V.dn_tiles = 0;
             if (g.dn_r) {
                 V.dn_a = reinterpret_cast<uint16_t *>(sp); sp += al(2ull * g.n);
@@ -436,10 +441,12 @@ void build_header(seg_ctx *ctx, Batch &b) {
                 V.raw = V.dn_out;  // the smoothing reads the denoised image
                 const uint64_t w = 2ull * g.dn_r + 1;
                 V.dn_mul = (uint32_t)(((1ull << 32) + w - 1) / w);
-                V.dn_n[0] = box_lines_items(g.rows, g.X, DN_CHUNK_X);
-                V.dn_n[1] = box_lines_items((uint64_t)g.X * g.Z, g.Y, DN_CHUNK);
-                V.dn_n[2] = box_lines_items((uint64_t)g.X * g.Y, g.Z, DN_CHUNK);
-                dn_classes |= g.dn_r <= 4u ? 1u : (g.dn_r <= 8u ? 2u : 4u);
+                V.dn_ring = box_rings(g.X, g.Z, g.dn_r, dn_all, ctx->sms);
+                for (int a = 0; a < 3; ++a) {
+                    const bool ring = (V.dn_ring >> a & 1u) != 0u;
+                    V.dn_n[a] = (uint32_t)box_items(a, ring, g.X, g.Y, g.Z);
+                    dn_routes |= 1u << box_route_bit(a, ring ? box_class(g.dn_r) : 3);
+                }
                 V.dn_tiles = (uint32_t)(cdiv(g.X, MED_TILE_X) * cdiv(g.Y, MED_TILE_Y) * cdiv(g.Z, MED_TILE_Z));
             }
             V.dn_base0 = dn[0];
@@ -606,7 +613,7 @@ void build_header(seg_ctx *ctx, Batch &b) {
     h->dn_items[1] = dn[1];
     h->dn_items[2] = dn[2];
     h->dn_tiles = dnt;
-    b.dn_classes = dn_classes;
+    b.dn_routes = dn_routes;
     h->cl_items = cl;
     for (int k = 0; k < DT_NK; ++k) h->dt_items[k] = dtb[k];
     h->mrf_tiles = mrft;
@@ -702,7 +709,7 @@ int launch_batch(seg_ctx *ctx, Batch &b) {
     }
     ctx->plan.rows = s.h_hdr->fs_tiles > 0;
     ctx->plan.tiles = s.h_hdr->ntiles > 0;
-    ctx->plan.denoise = b.dn_classes;
+    ctx->plan.denoise = b.dn_routes;
     ctx->plan.closing = s.h_hdr->cl_items > 0;
     ctx->plan.distance = false;
     for (int k = 0; k < DT_NK; ++k) ctx->plan.distance |= s.h_hdr->dt_items[k] > 0;
