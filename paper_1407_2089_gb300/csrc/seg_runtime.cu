@@ -39,6 +39,19 @@ inline uint64_t cdiv(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
 
 struct Batch;
 
+// Where the smoothed image of a volume lives until its threshold: the kept
+// image (SEG_KEEP_SMOOTHED); the label image, unused until the label kernel, for
+// rows of X % 8 != 0 voxels, padded there to whole octets (2 bytes a voxel of at
+// most 2 X) so that the smoothing stores and the threshold loads 16 bytes at a
+// time; else scratch.
+enum class SmoothAt { kept, labels, scratch };
+
+SmoothAt smooth_at(uint32_t X, uint32_t rows, bool keep) {
+    if (keep) return SmoothAt::kept;
+    const uint32_t p = (X + 7u) / 8u * 8u;
+    return X % 8u != 0u && p <= 2u * X && (uint64_t)p * rows < (1ull << 32) ? SmoothAt::labels : SmoothAt::scratch;
+}
+
 // Geometry and footprint of one channel of a request.
 struct VolGeom {
     uint32_t X, Y, Z, W, rows, nrt;
@@ -48,6 +61,7 @@ struct VolGeom {
     uint32_t dt_w[3];   // distance-map weights, {0, 0, 0} = off
     uint32_t mrf_max;   // MRF denoise step limit, 0 = off
     uint64_t n, r_cap, k_cap;
+    SmoothAt smooth;
     size_t scratch;  // bytes of per-batch scratch for this volume-channel
 };
 
@@ -73,7 +87,7 @@ DtPath dt_path(uint32_t X, uint32_t Y, uint32_t Z) {
 }
 
 VolGeom geom(seg_dims d, uint32_t min_volume, uint32_t dn_r, uint32_t cl_r, const uint32_t *dt_w,
-             uint32_t mrf_max) {
+             uint32_t mrf_max, bool keep_smoothed) {
     VolGeom g;
     g.X = d.x; g.Y = d.y; g.Z = d.z;
     g.W = (uint32_t)cdiv(d.x, 32);
@@ -86,7 +100,9 @@ VolGeom geom(seg_dims d, uint32_t min_volume, uint32_t dn_r, uint32_t cl_r, cons
     uint64_t kc = cdiv(d.x, 2) * cdiv(d.y, 2) * cdiv(d.z, 2);
     if (min_volume > 1) kc = std::min<uint64_t>(kc, g.n / min_volume + 1);
     g.k_cap = std::max<uint64_t>(kc, 1);
-    g.scratch = al(4ull * HIST_BINS) + al(2ull * g.n) + al(2ull * g.rows * g.W) + al(4ull * g.rows * g.W) +
+    g.smooth = smooth_at(d.x, g.rows, keep_smoothed);
+    g.scratch = al(4ull * HIST_BINS) + (g.smooth == SmoothAt::scratch ? al(2ull * g.n) : 0) +
+                al(2ull * g.rows * g.W) + al(4ull * g.rows * g.W) +
                 al(4ull * (g.rows + 1)) +
                 al(4ull * g.rows) + 2 * al(4ull * g.nrt) + 3 * al(4ull * g.r_cap);
     g.dn_r = dn_r;
@@ -517,20 +533,14 @@ void build_header(seg_ctx *ctx, Batch &b) {
                 }
             }
             V.hist = reinterpret_cast<uint32_t *>(sp); sp += al(4ull * HIST_BINS);
-            V.smooth = reinterpret_cast<uint16_t *>(sp); sp += al(2ull * g.n);
             V.sm_pitch = g.X;
-            if (r->smoothed(c)) {
+            if (g.smooth == SmoothAt::kept) {
                 V.smooth = r->smoothed(c);
-            } else if (g.X % 8u != 0u) {
-                // rows of X % 8 != 0 voxels go into the label image, unused
-                // until the label kernel, with rows padded to whole octets
-                // (2 bytes a voxel of at most 2 X), so that the smoothing
-                // stores and the threshold loads 16 bytes at a time
-                const uint32_t p = (g.X + 7u) / 8u * 8u;
-                if (p <= 2u * g.X && (uint64_t)p * g.rows < (1ull << 32)) {
-                    V.smooth = reinterpret_cast<uint16_t *>(V.labels);
-                    V.sm_pitch = p;
-                }
+            } else if (g.smooth == SmoothAt::labels) {
+                V.smooth = reinterpret_cast<uint16_t *>(V.labels);
+                V.sm_pitch = (g.X + 7u) / 8u * 8u;
+            } else {
+                V.smooth = reinterpret_cast<uint16_t *>(sp); sp += al(2ull * g.n);
             }
             V.wmax = reinterpret_cast<uint16_t *>(sp); sp += al(2ull * g.rows * g.W);
             V.mask = reinterpret_cast<uint32_t *>(sp); sp += al(4ull * g.rows * g.W);
@@ -1050,6 +1060,7 @@ int seg_submit_volume(seg_ctx *ctx, const uint16_t *voxels, int on_device, seg_d
     r->dims = dims;
     r->C = channels;
     r->minvol.resize(channels);
+    const bool keep = (ctx->cfg.flags & SEG_KEEP_SMOOTHED) != 0;
     for (uint32_t c = 0; c < channels; ++c) {
         uint32_t m = per_channel ? per_channel[c].min_volume_voxels : 30u;
         const uint32_t dr = per_channel ? per_channel[c].denoise_radius : 0u;
@@ -1070,7 +1081,7 @@ int seg_submit_volume(seg_ctx *ctx, const uint16_t *voxels, int on_device, seg_d
         const uint32_t mi = per_channel ? per_channel[c].mrf_iterations : 0u;
         if (mi > MRF_MAX_ITER || (mi && dr)) return SEG_EINVAL;
         r->minvol[c] = m ? m : 1u;  // a cell has at least one voxel
-        r->g.push_back(geom(dims, r->minvol[c], dr, cr, dw, mi));
+        r->g.push_back(geom(dims, r->minvol[c], dr, cr, dw, mi, keep));
     }
     {
         uint64_t rl = 0;
@@ -1088,7 +1099,7 @@ int seg_submit_volume(seg_ctx *ctx, const uint16_t *voxels, int on_device, seg_d
     r->errbits.assign(channels, 0);
     r->owns_input = host_in;
     if (!host_in) r->user_dev = voxels;
-    layout_request(*r, (ctx->cfg.flags & SEG_KEEP_SMOOTHED) != 0);
+    layout_request(*r, keep);
     if (r->persist + r->scratch > ctx->budget) return SEG_ETOOBIG;
     cudaSetDevice(ctx->device);
     if (cudaEventCreateWithFlags(&r->done_ev, cudaEventDisableTiming) != cudaSuccess) {
