@@ -17,8 +17,8 @@
 // of them; a chunk inside a line starts 3r positions early with empty rings,
 // which fill by the time its first output is due.
 //
-// Bound by the latency of its loads along x and y (IPC 1.6 and 1.8 of 4, long
-// scoreboard first), between that and instruction issue along z (2.2).  4 volumes
+// Bound by the latency of its loads along x and y (IPC 1.8 and 1.9 of 4,
+// long scoreboard first), between that and instruction issue along z (2.3).  4 volumes
 // of 512 x 512 x 64, r = 8: x 238 -> 223, y 153 -> 101, z 214 -> 147 us against the
 // other form, three passes through shared memory with a barrier each (k_box3),
 // which is the faster one for small batches and large radii.  Chunks of 256

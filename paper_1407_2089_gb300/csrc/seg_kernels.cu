@@ -2601,9 +2601,10 @@ __global__ void k_gather_stat(const BatchHdr *__restrict__ h, uint32_t *out) {
 // the smoothing reads.  Each thread takes two neighbouring voxels along x:
 // the comparator networks run on 16-bit halves of 32-bit words (packed min
 // and max), and the pairs of a 3x3 row are two aligned shared-memory words
-// and one byte permutation of them.  Bound by the min / max pipe: 411 us for
-// four volumes of 512 x 512 x 64, 462 with a median network over three sorted
-// lists per voxel.
+// and one byte permutation of them.  Bound by the pipe that takes the packed
+// minima and maxima (70 % busy at IPC 2.4 of 4, its throttle among the first
+// stalls; 144 thread instructions per voxel): 411 us for four volumes of 512 x
+// 512 x 64, 462 with a median network over three sorted lists per voxel.
 constexpr int MED_TX = 32, MED_TY = 8, MED_TZ = 8;  // threads along x and y; planes per tile
 static_assert(2 * MED_TX == MED_TILE_X && MED_TY == MED_TILE_Y && MED_TZ == MED_TILE_Z && MED_TZ % 2 == 0, "median tile");
 
@@ -3264,8 +3265,9 @@ __device__ __forceinline__ void mrf_planes(const VolDev &V, uint32_t o0, uint32_
 // extra plane on either side.  Splitting z keeps all multiprocessors busy for
 // a single volume (a 512 x 512 x 64 volume has only 128 tiles).
 //
-// Bound by instruction issue (about 15 per voxel), near its traffic of 6 bytes
-// per voxel: 89 us a step for four 512 x 512 x 64 volumes (4.5 TB/s, 0.67 of
+// 27 thread instructions per voxel at IPC 2.2 of 4, a third of the warps resident
+// and long scoreboard the first stall: bound by the latency of its loads as much
+// as by issue, near its traffic of 6 bytes per voxel: 89 us a step for four 512 x 512 x 64 volumes (4.5 TB/s, 0.67 of
 // the measured copy rate) and 24 us for one, where whole-z tiles of 256 x 8
 // voxels with scalar votes took 277 and 115 us.  Three blocks per
 // multiprocessor: two take 114 us, four 27 us for the one volume.
